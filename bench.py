@@ -45,7 +45,7 @@ MEDIUM_WORKLOAD = "campus_200k_tris_400x200_rays_5_bounces_2000_bins"
 L2_FLUSH_BYTES = 256 << 20
 METRIC = "Mrays/s (all bounces) & scans/s on 1 GB300; p50/p99 served scan latency"
 RAY_IO_BYTES = 48 + 16          # ray record read + hit record written per closest-hit query
-NODE_BYTES, TRI_BYTES = 64, 48  # BVH node and triangle record
+NODE_BYTES, TRI_BYTES = 32, 48  # BVH node and triangle record
 L2_FLUSH_NOTE = "flushed between steps (256 MiB write, outside the timed events)"
 ORDER_DEFAULT = "queue"         # the library's default query order (rr_batch_config.query_order)
 

@@ -377,11 +377,11 @@ int rr_scan_batch_async(rr_scene* scene, uint32_t n, const rr_pose* poses, const
    trace_blocks_per_sm  resident trace blocks per SM (0: the occupancy maximum)
    use_graph            1: each launch sequence is captured once in a CUDA
                         graph and replayed while its arguments stay the same
-   node_format          RR_NODES_BINARY (default): traverse the binary LBVH
-                        with float boxes; RR_NODES_WIDE8: the 8-wide BVH with
-                        8-bit quantised child boxes.  Both give the same
-                        closest hit for every query (the quantised boxes are
-                        rounded outward onto exact float bounds).
+   node_format          RR_NODES_BINARY (default): traverse the binary LBVH,
+                        its child boxes on a 16-bit grid over the scene;
+                        RR_NODES_WIDE8: the 8-wide BVH with 8-bit child boxes
+                        on a grid per node.  Both give the same closest hit
+                        for every query (the boxes are rounded outward).
    refill_threshold     the query kernels keep their lanes busy by handing a
                         warp's idle lanes new queries once at least this many
                         of its 32 lanes are idle (1..32; 0 = 16)

@@ -526,14 +526,15 @@ int rr_scene_export_bvh(const rr_scene* s, uint32_t* morton, uint32_t* perm, uin
   if (T > 1 && children) RR_CHECK_CUDA(cudaMemcpy(children, s->d_child, (T - 1) * 8, cudaMemcpyDeviceToHost), "export");
   if (parents) RR_CHECK_CUDA(cudaMemcpy(parents, s->d_parent, (2 * T - 1) * 4, cudaMemcpyDeviceToHost), "export");
   if (T > 1 && boxes) {
-    std::vector<float4> nodes((T - 1) * 4);
-    RR_CHECK_CUDA(cudaMemcpy(nodes.data(), s->d_nodes, nodes.size() * sizeof(float4), cudaMemcpyDeviceToHost),
-                  "export");
-    for (size_t i = 0; i + 1 < T; ++i) {
-      const float4 n0 = nodes[4 * i], n1 = nodes[4 * i + 1], n2 = nodes[4 * i + 2];
-      float* b = boxes + 12 * i;
-      const float v[12] = {n0.x, n0.z, n2.x, n0.y, n0.w, n2.y, n1.x, n1.z, n2.z, n1.y, n1.w, n2.w};
-      memcpy(b, v, sizeof v);
+    // the float boxes of the build (the traversal's nodes hold them rounded outward to a grid)
+    std::vector<uint32_t> child((T - 1) * 2);
+    std::vector<float> nbox((2 * T - 1) * 6);
+    RR_CHECK_CUDA(cudaMemcpy(child.data(), s->d_child, child.size() * 4, cudaMemcpyDeviceToHost), "export");
+    RR_CHECK_CUDA(cudaMemcpy(nbox.data(), s->d_nbox, nbox.size() * 4, cudaMemcpyDeviceToHost), "export");
+    for (size_t i = 0; i < 2 * (T - 1); ++i) {
+      const uint32_t c = child[i];
+      const size_t slot = (c & rr::kLeafBit) ? T - 1 + (c & ~rr::kLeafBit) : c;
+      memcpy(boxes + 6 * i, &nbox[6 * slot], 6 * sizeof(float));
     }
   }
   return RR_OK;

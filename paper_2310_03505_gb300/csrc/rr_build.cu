@@ -14,10 +14,9 @@
 // plus the per-material lobe table of Eq. 5 used by the beam window (Eq. 4).
 //
 // The hierarchy is a binary BVH with one triangle per leaf.  Internal node i
-// is stored as four float4 (Aila & Laine, HPG 2009 layout):
-//   n0 = (c0.lo.x, c0.hi.x, c0.lo.y, c0.hi.y)   n1 = same for child 1
-//   n2 = (c0.lo.z, c0.hi.z, c1.lo.z, c1.hi.z)   n3 = (child0, child1, 0, 0)
-// with a child reference i for internal node i and j | 0x80000000 for leaf j.
+// is stored in 32 bytes: both child boxes rounded outward to a 16-bit grid
+// over the scene, and the child references (layout: kNodeWords); the float
+// boxes stay in nbox.
 // Leaves are the triangles in sorted order: tri[3j..3j+2] = v0, v1, v2 with
 // v0.w = original triangle id, v1.w = material id (bit patterns).
 #include <algorithm>
@@ -63,15 +62,22 @@ __device__ __forceinline__ void st_release_u32(uint32_t* p, uint32_t v) {
 
 // ---------------------------------------------------------------------------
 // a1: validation, centroids and centroid bounds
-// misc[0..2] = encoded min xyz, misc[3..5] = encoded max xyz, misc[6] = error
+// misc[0..2] = ~encoded min xyz of the centroids, misc[3..5] = encoded max
+// xyz, misc[6] = error, misc[8..13] = the same bounds of the vertices (each a
+// maximum, so that all start from zero)
 __global__ void k_ingest(const float* __restrict__ vtx, const uint32_t* __restrict__ idx,
                          const uint16_t* __restrict__ mat_id, uint32_t nv, uint32_t nt, uint32_t nm,
                          float4* __restrict__ centroid, uint32_t* __restrict__ misc) {
-  __shared__ float s_lo[3][32], s_hi[3][32];
+  __shared__ float s_lo[6][32], s_hi[6][32];
   const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-  float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
+  float lo[6], hi[6];   // centroid, vertices
+  for (int k = 0; k < 6; ++k) {
+    lo[k] = INFINITY;
+    hi[k] = -INFINITY;
+  }
   if (i < nt) {
     uint32_t err = 0;
+    float vlo[3] = {0.f, 0.f, 0.f}, vhi[3] = {0.f, 0.f, 0.f};
     const uint32_t a = idx[3 * i], b = idx[3 * i + 1], c = idx[3 * i + 2];
     if (a >= nv || b >= nv || c >= nv) err |= 1u;
     if (mat_id[i] >= nm) err |= 2u;
@@ -81,17 +87,23 @@ __global__ void k_ingest(const float* __restrict__ vtx, const uint32_t* __restri
         const float x0 = vtx[3 * a + k], x1 = vtx[3 * b + k], x2 = vtx[3 * c + k];
         if (!isfinite(x0) || !isfinite(x1) || !isfinite(x2)) err |= kErrBadVertex;
         cen[k] = (x0 + x1 + x2) / 3.0f;
+        vlo[k] = fminf(fminf(x0, x1), x2);
+        vhi[k] = fmaxf(fmaxf(x0, x1), x2);
       }
     }
     if (err) {
       atomicOr(&misc[6], err);
     } else {
-      for (int k = 0; k < 3; ++k) lo[k] = hi[k] = cen[k];
+      for (int k = 0; k < 3; ++k) {
+        lo[k] = hi[k] = cen[k];
+        lo[3 + k] = vlo[k];
+        hi[3 + k] = vhi[k];
+      }
     }
     centroid[i] = make_float4(cen[0], cen[1], cen[2], 0.f);
   }
   // warp then block reduction of the bounds
-  for (int k = 0; k < 3; ++k) {
+  for (int k = 0; k < 6; ++k) {
     for (int off = 16; off > 0; off >>= 1) {
       lo[k] = fminf(lo[k], __shfl_xor_sync(0xFFFFFFFFu, lo[k], off));
       hi[k] = fmaxf(hi[k], __shfl_xor_sync(0xFFFFFFFFu, hi[k], off));
@@ -99,21 +111,22 @@ __global__ void k_ingest(const float* __restrict__ vtx, const uint32_t* __restri
   }
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   if (lane == 0)
-    for (int k = 0; k < 3; ++k) {
+    for (int k = 0; k < 6; ++k) {
       s_lo[k][warp] = lo[k];
       s_hi[k][warp] = hi[k];
     }
   __syncthreads();
   if (warp == 0) {
-    for (int k = 0; k < 3; ++k) {
+    for (int k = 0; k < 6; ++k) {
       float l = lane < nw ? s_lo[k][lane] : INFINITY, h = lane < nw ? s_hi[k][lane] : -INFINITY;
       for (int off = 16; off > 0; off >>= 1) {
         l = fminf(l, __shfl_xor_sync(0xFFFFFFFFu, l, off));
         h = fmaxf(h, __shfl_xor_sync(0xFFFFFFFFu, h, off));
       }
       if (lane == 0 && l <= h) {
-        atomicMin(&misc[k], enc_f(l));
-        atomicMax(&misc[3 + k], enc_f(h));
+        const int o = k < 3 ? k : 8 + (k - 3);
+        atomicMax(&misc[o], ~enc_f(l));
+        atomicMax(&misc[o + 3], enc_f(h));
       }
     }
   }
@@ -130,16 +143,32 @@ __device__ __forceinline__ uint32_t spread3(uint32_t v) {
 
 // a2: code = x9 y9 z9 x8 y8 z8 ... x0 y0 z0 of the quantised centroid
 // also counts the first sort pass's digits per tile (hist0, zeroed before)
-__global__ void k_morton(const float4* __restrict__ centroid, const uint32_t* __restrict__ misc, uint32_t nt,
+// and lays the grid of the binary nodes over the vertex bounds
+__global__ void k_morton(const float4* __restrict__ centroid, uint32_t* __restrict__ misc, uint32_t nt,
                          uint32_t* __restrict__ keys, uint32_t* __restrict__ vals, uint32_t tiles,
                          uint32_t* __restrict__ hist0) {
   const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= nt) return;
+  if (i == 0) {
+    // lower bound at F = 0.501, upper bound at 1.997: a thousandth of slack on
+    // either side for the outward rounding.  The scale is at least 2^-11 of
+    // the coordinates, so that rounding the base moves no bound out of range.
+    float* fr = reinterpret_cast<float*>(misc + kFrameWord);
+    for (int k = 0; k < 3; ++k) {
+      float lo = dec_f(~misc[8 + k]), hi = dec_f(misc[11 + k]);
+      if (!(lo <= hi)) lo = hi = 0.0f;   // no valid triangle: the build is reported as failed
+      const float scale =
+          fmaxf(fminf(fmaxf((hi - lo) * (1.0f / 1.496f), 0x1p-11f * fmaxf(fabsf(lo), fabsf(hi))), 1e37f), 1e-30f);
+      fr[k] = lo - 0.501f * scale;
+      fr[4 + k] = scale;
+    }
+    fr[3] = fr[7] = 0.0f;
+  }
   const float4 c = centroid[i];
   const float cc[3] = {c.x, c.y, c.z};
   uint32_t q[3];
   for (int k = 0; k < 3; ++k) {
-    const float lo = dec_f(misc[k]), hi = dec_f(misc[3 + k]);
+    const float lo = dec_f(~misc[k]), hi = dec_f(misc[3 + k]);
     const float ext = hi - lo;
     const float x = ext > 0.0f ? (cc[k] - lo) / ext : 0.0f;
     q[k] = (uint32_t)fminf(floorf(x * 1024.0f), 1023.0f);
@@ -524,6 +553,32 @@ __device__ __forceinline__ uint32_t classify_member(uint32_t c, const uint32_t* 
   return (tris <= kGroupMax && c < (1u << kGroupShift)) ? (kGroupBit | (tris << kGroupShift) | c) : c;
 }
 
+// grid codes of a lower and an upper bound: f = (x - base) / scale errs by at
+// most a few units of 2^-23 (f < 2), the margin 2^-20 covers that, then the
+// low byte is cut off downward or upward
+__device__ __forceinline__ uint32_t grid_lo(float x, float base, float inv) {
+  const float f = fminf(fmaxf((x - base) * inv - 0x1p-20f, 0.5f), 1.9999f);
+  return (__float_as_uint(f) >> 8) & 0xFFFFu;
+}
+__device__ __forceinline__ uint32_t grid_hi(float x, float base, float inv) {
+  const float f = fminf(fmaxf((x - base) * inv + 0x1p-20f, 0.5f), 1.9999f);
+  return ((__float_as_uint(f) + 0xFFu) >> 8) & 0xFFFFu;
+}
+
+// binary node p: boxes b0, b1 (lo xyz, hi xyz) of its children c0, c1
+__device__ __forceinline__ void write_node(uint4* __restrict__ nodes, size_t p, const float* __restrict__ frame,
+                                           const float* b0, const float* b1, uint32_t c0, uint32_t c1) {
+  uint32_t w[6];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const float base = __ldg(frame + k), inv = 1.0f / __ldg(frame + 4 + k);
+    w[k] = grid_lo(b0[k], base, inv) | grid_hi(b0[3 + k], base, inv) << 16;
+    w[3 + k] = grid_lo(b1[k], base, inv) | grid_hi(b1[3 + k], base, inv) << 16;
+  }
+  nodes[kNodeWords * p] = make_uint4(w[0], w[1], w[2], w[3]);
+  nodes[kNodeWords * p + 1] = make_uint4(w[4], w[5], c0, c1);
+}
+
 // a5: each leaf walks to the root; at every internal node the first arrival
 // stops and the second merges both child boxes (they are final by then).
 // The walker carries the box of the child it comes from, so it reads only
@@ -537,7 +592,8 @@ constexpr int kRefitBlock = 256;
 __global__ void __launch_bounds__(kRefitBlock) k_refit(uint32_t n, const uint32_t* __restrict__ child,
                                                        const uint32_t* __restrict__ parent,
                                                        const uint2* __restrict__ range, uint32_t* __restrict__ visit,
-                                                       float* __restrict__ nbox, float4* __restrict__ nodes) {
+                                                       float* __restrict__ nbox, uint4* __restrict__ nodes,
+                                                       const float* __restrict__ frame) {
   __shared__ float s_box[2][kRefitBlock][6];   // [0] the block's leaves, [1] its local internal nodes
   __shared__ uint32_t s_visit[kRefitBlock];
   const uint32_t base = blockIdx.x * kRefitBlock, end = min(base + kRefitBlock, n);
@@ -581,11 +637,7 @@ __global__ void __launch_bounds__(kRefitBlock) k_refit(uint32_t n, const uint32_
       b0[k] = first_is_own ? own[k] : sb[k];
       b1[k] = first_is_own ? sb[k] : own[k];
     }
-    float4* nd = nodes + 4 * (size_t)p;
-    nd[0] = make_float4(b0[0], b0[3], b0[1], b0[4]);
-    nd[1] = make_float4(b1[0], b1[3], b1[1], b1[4]);
-    nd[2] = make_float4(b0[2], b0[5], b1[2], b1[5]);
-    nd[3] = make_float4(__uint_as_float(c0), __uint_as_float(c1), 0.f, 0.f);
+    write_node(nodes, p, frame, b0, b1, c0, c1);
     float* bp = nbox + 6 * (size_t)p;
     for (int k = 0; k < 3; ++k) {
       own[k] = fminf(b0[k], b1[k]);
@@ -778,7 +830,8 @@ struct TopArgs {
   uint4* small;           // [C - 1] warp tasks (2 to kTopSmall clusters)
   uint32_t* ctr;          // kCtr*
   uint32_t* cb;           // [T - 1][6] centroid bounds (encoded) of the block task at each node slot
-  float4* nodes;
+  uint4* nodes;
+  const float* frame;     // grid of the binary nodes
   uint32_t* child;
   uint32_t* parent;
   float* nbox;
@@ -889,11 +942,7 @@ __device__ Split warp_best_split(const uint32_t* bins, int lane) {
 // the node of a task: child boxes (lo xyz, hi xyz) and references
 __device__ __forceinline__ void write_top_node(const TopArgs& a, uint32_t slot, const float (&bx)[2][6],
                                                const uint32_t (&ref)[2]) {
-  float4* nd = a.nodes + 4 * (size_t)slot;
-  nd[0] = make_float4(bx[0][0], bx[0][3], bx[0][1], bx[0][4]);
-  nd[1] = make_float4(bx[1][0], bx[1][3], bx[1][1], bx[1][4]);
-  nd[2] = make_float4(bx[0][2], bx[0][5], bx[1][2], bx[1][5]);
-  nd[3] = make_float4(__uint_as_float(ref[0]), __uint_as_float(ref[1]), 0.f, 0.f);
+  write_node(a.nodes, slot, a.frame, bx[0], bx[1], ref[0], ref[1]);
   a.child[2 * slot] = ref[0];
   a.child[2 * slot + 1] = ref[1];
   for (int side = 0; side < 2; ++side) a.parent[node_slot(ref[side], a.n)] = slot;
@@ -1915,7 +1964,7 @@ cudaError_t build_alloc(rr_scene* s) {
   RR_TRY(alloc((void**)&s->d_lut_cells, M * kLutCells * sizeof(float)));
   RR_TRY(alloc((void**)&s->d_lobe_kind, M * sizeof(uint8_t)));
   RR_TRY(alloc((void**)&s->d_tri, (kTriCopies * 3 + 1) * T * sizeof(float4)));
-  RR_TRY(alloc((void**)&s->d_nodes, (T > 1 ? T - 1 : 0) * 4 * sizeof(float4)));
+  RR_TRY(alloc((void**)&s->d_nodes, (T > 1 ? T - 1 : 0) * kNodeWords * sizeof(uint4)));
   RR_TRY(alloc((void**)&s->d_centroid, T * sizeof(float4)));
   for (int k = 0; k < 2; ++k) {
     RR_TRY(alloc((void**)&s->d_keys[k], T * sizeof(uint32_t)));
@@ -1928,8 +1977,8 @@ cudaError_t build_alloc(rr_scene* s) {
   RR_TRY(alloc((void**)&s->d_child, (T > 1 ? T - 1 : 1) * 2 * sizeof(uint32_t)));
   RR_TRY(alloc((void**)&s->d_nbox, (T ? 2 * T - 1 : 1) * 6 * sizeof(float)));
   RR_TRY(alloc((void**)&s->d_visit, (T > 1 ? T - 1 : 1) * sizeof(uint32_t)));
-  RR_TRY(alloc((void**)&s->d_misc, 8 * sizeof(uint32_t)));
-  RR_TRY(cudaMemset(s->d_misc, 0, 8 * sizeof(uint32_t)));   // status of an empty scene: no error
+  RR_TRY(alloc((void**)&s->d_misc, kMiscWords * sizeof(uint32_t)));
+  RR_TRY(cudaMemset(s->d_misc, 0, kMiscWords * sizeof(uint32_t)));   // status of an empty scene: no error
   RR_TRY(alloc((void**)&s->d_range, (T > 1 ? T - 1 : 1) * sizeof(uint2)));
   // wide BVH: at most T - 1 wide nodes (each owns a distinct binary internal node)
   s->wcap = T > 1 ? (uint32_t)(T - 1) : 1u;
@@ -2014,6 +2063,7 @@ static cudaError_t build_sah_top(rr_scene* s, cudaStream_t st) {
   a.ctr = s->d_top_ctr;
   a.cb = s->d_top_cb;
   a.nodes = s->d_nodes;
+  a.frame = reinterpret_cast<const float*>(s->d_misc + kFrameWord);
   a.child = s->d_child;
   a.parent = s->d_parent;
   a.nbox = s->d_nbox;
@@ -2035,9 +2085,8 @@ static cudaError_t build_sah_top(rr_scene* s, cudaStream_t st) {
 
 cudaError_t build_lbvh(rr_scene* s, cudaStream_t st, bool with_depth) {
   const uint32_t n = s->nt;
-  // bounds reset: min slots to all ones, max slots, error and depth to zero
-  RR_TRY(cudaMemsetAsync(s->d_misc, 0xFF, 3 * sizeof(uint32_t), st));
-  RR_TRY(cudaMemsetAsync(s->d_misc + 3, 0, 5 * sizeof(uint32_t), st));
+  // bounds, error and depth start from zero
+  RR_TRY(cudaMemsetAsync(s->d_misc, 0, kFrameWord * sizeof(uint32_t), st));
   if (n == 0) return cudaSuccess;
   const int B = 256;
   const uint32_t g = (n + B - 1) / B;
@@ -2082,7 +2131,8 @@ cudaError_t build_lbvh(rr_scene* s, cudaStream_t st, bool with_depth) {
                                                 s->d_range);
     RR_TRY(cudaGetLastError());
     k_refit<<<(n + kRefitBlock - 1) / kRefitBlock, kRefitBlock, 0, st>>>(n, s->d_child, s->d_parent, s->d_range,
-                                                                           s->d_visit, s->d_nbox, s->d_nodes);
+                                                                           s->d_visit, s->d_nbox, s->d_nodes,
+                                                                           reinterpret_cast<const float*>(s->d_misc + kFrameWord));
     RR_TRY(cudaGetLastError());
     if (sah_top) RR_TRY(build_sah_top(s, st));
     if (with_depth) {

@@ -113,6 +113,22 @@ struct ScanCounters {
 // triangle.
 constexpr int kWideNodeWords = 5;
 
+// Binary BVH node, two uint4 (32 bytes, read with one 256-bit load):
+//   (box0 x, box0 y, box0 z, box1 x) (box1 y, box1 z, child0, child1)
+// a child reference is i for internal node i, j | kLeafBit for leaf j.  A box
+// word holds an axis's lower bound in its low 16 bits and the upper bound in
+// its high 16 bits, as codes q of a grid over the whole scene: code q stands
+// for the float F = bits 0x3F000000 | q << 8 of [0.5, 2) and the plane at
+// base + F scale (the frame).  Codes are rounded outward, so a decoded box
+// contains the child's float box.  The float boxes took 64 bytes; what the
+// closest-hit query pays for is the fetch (2 x 128 bits against 4, and half
+// the L1 and L2 footprint), and one byte permutation per plane picks the near
+// or far plane and decodes it, where the float form needed a min and a max.
+constexpr int kNodeWords = 2;
+// The grid of a scene's binary nodes, two float4: (base x, y, z, 0), (scale x, y, z, 0)
+constexpr int kFrameWord = 16;        // its place in the build status words (rr_scene::d_misc)
+constexpr int kMiscWords = 24;        // 0..5 centroid bounds, 6 error bits, 7 depth, 8..13 vertex bounds, 16..23 the frame
+
 // Return record key: global image column (scan's first column + azimuth)
 // and range bin.  Records of one bounce are in column order.
 constexpr int kBinBits = 14;                       // n_bins <= RR_MAX_BINS = 2^14
@@ -149,7 +165,8 @@ struct ScanArgs {
                              // the coordinates rotated by r (tri_rotate), so copy 0 is (x, y, z); then [T]
                              // (unit geometric normal, material bits) at tri + 3 tri_copy
   size_t tri_copy;           // float4s from one rotated copy to the next (3 T)
-  const float4* nodes;       // [T-1][4] Aila-Laine layout
+  const uint4* nodes;        // binary: [T-1][kNodeWords], wide: [.][kWideNodeWords]
+  const float4* frame;       // [2] grid of the binary nodes' boxes
   const MatDev* mats;
   const float4* lut;         // [M][kLutCells + 1]: (G(x_k), Gc(x_k), cos^C(x_k), 0)
   uint32_t n_tris, n_mats;

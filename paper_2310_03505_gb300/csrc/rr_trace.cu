@@ -29,7 +29,7 @@
 namespace rr {
 
 constexpr int kShadeBlock = 256;
-constexpr float kBoxInflate = 1.00000036f;  // 1 + 2 gamma_3 (robust slab test, Ize 2013)
+constexpr float kBoxInflate = 1.00000036f;  // 1 + 2 gamma_3 (robust slab test, Ize 2013): wide nodes
 
 // ---------------------------------------------------------------------------
 // beam axis angle 2 pi a / n with an exact quadrant reduction; returns (cos, sin)
@@ -161,6 +161,24 @@ __device__ __forceinline__ float woop_hit(const WoopRay& w, float3 v0, float3 v1
   return T / det;
 }
 
+// Selectors of a binary node's box word: __byte_perm(word, 0x3F000000, sel)
+// gives the float F of the lower / upper bound (kNodeWords); they differ in
+// the bits kSelFlip.
+constexpr uint32_t kSelLo = 0x7104u, kSelHi = 0x7324u, kSelFlip = 0x0220u;
+__device__ __forceinline__ float grid_plane(uint32_t word, uint32_t sel) {
+  return __uint_as_float(__byte_perm(word, 0x3F000000u, sel));
+}
+__device__ __forceinline__ float max3(float a, float b, float c) {
+  float d;
+  asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  return d;
+}
+__device__ __forceinline__ float min3(float a, float b, float c) {
+  float d;
+  asm("min.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  return d;
+}
+
 // ---------------------------------------------------------------------------
 // Resumable traversal.  A query (closest hit, or any hit for visibility) is
 // advanced one step at a time -- one node visit or one triangle test -- so
@@ -171,10 +189,10 @@ __device__ __forceinline__ float woop_hit(const WoopRay& w, float3 v0, float3 v1
 // lexicographically smallest.  Any hit: the first t_min < t < t_best.  The
 // leaf `skip` (the one the ray starts on) is never reported.
 struct Trav {
-  float3 c0, c1;        // slab offsets (trav_begin): binary nodes, of the lower / upper box planes;
-                        // wide nodes, of the near / far planes
+  float3 c0, c1;        // slab offsets of the near / far planes (trav_begin)
   WoopRay w;            // the watertight-test frame
-  float3 id;            // 1 / direction, zero components replaced by +-1e-30
+  float3 id;            // 1 / direction, zero components replaced by +-1e-30; binary nodes: times the grid scale
+  uint3 sel;            // binary: byte selectors that decode the near plane of a box word, per axis
   float t_min, t_best;
   uint32_t skip;
   uint32_t node;        // binary: next node; both: kNone once the query has ended
@@ -185,30 +203,44 @@ struct Trav {
   int sp;
 };
 
-__device__ __forceinline__ void trav_begin(Trav& s, float3 o, float3 d, float t_min, float t_best, uint32_t skip,
-                                           uint32_t n_tris, bool wide) {
+__device__ __forceinline__ void trav_begin(Trav& s, const ScanArgs& a, float3 o, float3 d, float t_min, float t_best,
+                                           uint32_t skip, bool wide) {
   s.w = make_woop(o, d);
   s.id = make_float3(1.0f / (fabsf(d.x) > 1e-30f ? d.x : copysignf(1e-30f, d.x)),
                      1.0f / (fabsf(d.y) > 1e-30f ? d.y : copysignf(1e-30f, d.y)),
                      1.0f / (fabsf(d.z) > 1e-30f ? d.z : copysignf(1e-30f, d.z)));
-  // Slab test with one fma per plane: plane b is reached at t = fma(b, id, c)
-  // with c = -(o id) -+ eps, where the robust form (b - o) id needs two
-  // operations.  The fma form errs against (b - o) id by at most u |o id|
-  // (o id rounded) + u |c| (c rounded) + u |t| (the fma itself), u = 2^-24.
-  // eps = 4 u |o id| moves every near plane down and every far plane up by
-  // more than the first two; the last is relative, like the errors of the
-  // robust form, and the far-plane inflation kBoxInflate covers it.  So a box
-  // the robust test accepts is accepted here too.
-  {
+  if (wide) {
+    // Slab test with one fma per plane: plane b is reached at t = fma(b, id, c)
+    // with c = -(o id) -+ eps, where the robust form (b - o) id needs two
+    // operations.  The fma form errs against (b - o) id by at most u |o id|
+    // (o id rounded) + u |c| (c rounded) + u |t| (the fma itself), u = 2^-24.
+    // eps = 4 u |o id| moves every near plane down and every far plane up by
+    // more than the first two; the last is relative, like the errors of the
+    // robust form, and the far-plane inflation kBoxInflate covers it.  So a box
+    // the robust test accepts is accepted here too.
     const float ox = __fmul_rn(o.x, s.id.x), oy = __fmul_rn(o.y, s.id.y), oz = __fmul_rn(o.z, s.id.z);
-    float ex = 0x1p-22f * fabsf(ox), ey = 0x1p-22f * fabsf(oy), ez = 0x1p-22f * fabsf(oz);
-    if (!wide) {   // the lower plane is the near one for a positive direction component
-      ex = copysignf(ex, s.id.x);
-      ey = copysignf(ey, s.id.y);
-      ez = copysignf(ez, s.id.z);
-    }
+    const float ex = 0x1p-22f * fabsf(ox), ey = 0x1p-22f * fabsf(oy), ez = 0x1p-22f * fabsf(oz);
     s.c0 = make_float3(-ox - ex, -oy - ey, -oz - ez);
     s.c1 = make_float3(-ox + ex, -oy + ey, -oz + ez);
+  } else {
+    // The same over grid planes base + F scale, F in [0.5, 2): t = fma(F, g, c)
+    // with g = scale id and c = (base - o) id.  Against the exact plane
+    // distance the rounded g errs by u |g| per unit of F, c by 3 u |c| and the
+    // fma by u |t|, and |t| <= 2 |g| + |c|: together with the relative
+    // far-plane inflation of the robust slab test (6 u |t|) less than
+    // eps = 24 u (2 |g| + |c|), which moves every near plane down and every
+    // far plane up, so that no inflation is left for the node visits.
+    const float4 base = __ldg(a.frame), scale = __ldg(a.frame + 1);
+    const float cx = __fmul_rn(base.x - o.x, s.id.x), cy = __fmul_rn(base.y - o.y, s.id.y),
+                cz = __fmul_rn(base.z - o.z, s.id.z);
+    s.sel = make_uint3(s.id.x < 0.0f ? kSelHi : kSelLo, s.id.y < 0.0f ? kSelHi : kSelLo,
+                       s.id.z < 0.0f ? kSelHi : kSelLo);
+    s.id = make_float3(scale.x * s.id.x, scale.y * s.id.y, scale.z * s.id.z);
+    const float ex = 0x1.8p-20f * (2.0f * fabsf(s.id.x) + fabsf(cx)),
+                ey = 0x1.8p-20f * (2.0f * fabsf(s.id.y) + fabsf(cy)),
+                ez = 0x1.8p-20f * (2.0f * fabsf(s.id.z) + fabsf(cz));
+    s.c0 = make_float3(cx - ex, cy - ey, cz - ez);
+    s.c1 = make_float3(cx + ex, cy + ey, cz + ez);
   }
   s.t_min = t_min;
   s.t_best = t_best;
@@ -223,9 +255,9 @@ __device__ __forceinline__ void trav_begin(Trav& s, float3 o, float3 d, float t_
     s.g_bits = (1u << 8) | (1u << s.oct);   // the root: internal slot 0 of a virtual group
     s.t_base = 0u;
     s.t_bits = 0u;
-    s.node = n_tris ? 0u : kNone;
+    s.node = a.n_tris ? 0u : kNone;
   } else {
-    s.node = n_tris == 0 ? kNone : (n_tris == 1 ? kLeafBit : 0u);
+    s.node = a.n_tris == 0 ? kNone : (a.n_tris == 1 ? kLeafBit : 0u);
   }
 }
 
@@ -255,65 +287,51 @@ __device__ __forceinline__ bool trav_tri(Trav& s, const ScanArgs& a, uint32_t j,
   return false;
 }
 
-// one step over the binary LBVH (both children tested, nearer first)
-template <bool kAny>
-__device__ __forceinline__ void step_binary(Trav& s, uint32_t* stack, const ScanArgs& a, uint32_t& n_nodes,
-                                            uint32_t& n_tris, bool count) {
-  const uint32_t node = s.node;
-  if (!(node & kLeafBit)) {
-    if (count) ++n_nodes;
-    ++s.visits;   // bounded where the query loop looks at its lanes
-    const float3 id = s.id, cl = s.c0, ch = s.c1;
-    const float4* np = a.nodes + 4 * (size_t)node;
-    const float4 n0 = __ldg(np), n1 = __ldg(np + 1), n2 = __ldg(np + 2), n3 = __ldg(np + 3);
-    // child 0
-    float t0 = fmaf(n0.x, id.x, cl.x), t1 = fmaf(n0.y, id.x, ch.x);
-    float lo0 = fminf(t0, t1), hi0 = fmaxf(t0, t1);
-    t0 = fmaf(n0.z, id.y, cl.y);
-    t1 = fmaf(n0.w, id.y, ch.y);
-    lo0 = fmaxf(lo0, fminf(t0, t1));
-    hi0 = fminf(hi0, fmaxf(t0, t1));
-    t0 = fmaf(n2.x, id.z, cl.z);
-    t1 = fmaf(n2.y, id.z, ch.z);
-    lo0 = fmaxf(fmaxf(lo0, fminf(t0, t1)), s.t_min);
-    hi0 = fminf(fminf(hi0, fmaxf(t0, t1)) * kBoxInflate, s.t_best);
-    // child 1
-    t0 = fmaf(n1.x, id.x, cl.x);
-    t1 = fmaf(n1.y, id.x, ch.x);
-    float lo1 = fminf(t0, t1), hi1 = fmaxf(t0, t1);
-    t0 = fmaf(n1.z, id.y, cl.y);
-    t1 = fmaf(n1.w, id.y, ch.y);
-    lo1 = fmaxf(lo1, fminf(t0, t1));
-    hi1 = fminf(hi1, fmaxf(t0, t1));
-    t0 = fmaf(n2.z, id.z, cl.z);
-    t1 = fmaf(n2.w, id.z, ch.z);
-    lo1 = fmaxf(fmaxf(lo1, fminf(t0, t1)), s.t_min);
-    hi1 = fminf(fminf(hi1, fmaxf(t0, t1)) * kBoxInflate, s.t_best);
-    const bool h0 = lo0 <= hi0, h1 = lo1 <= hi1;
-    const uint32_t c0 = __float_as_uint(n3.x), c1 = __float_as_uint(n3.y);
-    // the nearer hit child next, the farther one pushed when both are hit,
-    // else the next stack entry: selects and a predicated store instead of
-    // branches, so that the lanes of a warp take the same path here
-    const bool both = h0 && h1;
-    const bool first0 = !h1 || (h0 && lo0 <= lo1);
-    const uint32_t near = first0 ? c0 : c1, far = first0 ? c1 : c0;
-    const int sp = s.sp;
-    if (both && sp < kStack) stack[sp] = far;   // a predicated store: every local store costs an L2 sector
-    if (both && sp >= kStack) atomicOr(&a.ctr->error, kErrStack);
-    const int sp1 = sp + ((both && sp < kStack) ? 1 : 0);
-    if (h0 || h1) {
-      s.sp = sp1;
-      s.node = near;
-    } else {
-      s.node = sp1 ? stack[sp1 - 1] : kNone;
-      s.sp = sp1 ? sp1 - 1 : 0;
-    }
-    return;
-  } else if (trav_tri<kAny>(s, a, node & ~kLeafBit, n_tris, count)) {
-    s.node = kNone;
-    return;
+// Binary BVH: one inner node (both children tested, nearer first).
+__device__ __forceinline__ void step_inner(Trav& s, uint32_t* stack, const ScanArgs& a, uint32_t& n_nodes,
+                                           bool count) {
+  if (count) ++n_nodes;
+  ++s.visits;   // bounded where the query loop looks at its lanes
+  const uint4* np = a.nodes + kNodeWords * (size_t)s.node;
+  uint4 n0, n1;
+  asm("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+      : "=r"(n0.x), "=r"(n0.y), "=r"(n0.z), "=r"(n0.w), "=r"(n1.x), "=r"(n1.y), "=r"(n1.z), "=r"(n1.w)
+      : "l"(np));
+  const float3 g = s.id, cn = s.c0, cf = s.c1;
+  const uint3 sn = s.sel, sf = make_uint3(sn.x ^ kSelFlip, sn.y ^ kSelFlip, sn.z ^ kSelFlip);
+  const float lo0 = fmaxf(max3(fmaf(grid_plane(n0.x, sn.x), g.x, cn.x), fmaf(grid_plane(n0.y, sn.y), g.y, cn.y),
+                               fmaf(grid_plane(n0.z, sn.z), g.z, cn.z)), s.t_min);
+  const float hi0 = fminf(min3(fmaf(grid_plane(n0.x, sf.x), g.x, cf.x), fmaf(grid_plane(n0.y, sf.y), g.y, cf.y),
+                               fmaf(grid_plane(n0.z, sf.z), g.z, cf.z)), s.t_best);
+  const float lo1 = fmaxf(max3(fmaf(grid_plane(n0.w, sn.x), g.x, cn.x), fmaf(grid_plane(n1.x, sn.y), g.y, cn.y),
+                               fmaf(grid_plane(n1.y, sn.z), g.z, cn.z)), s.t_min);
+  const float hi1 = fminf(min3(fmaf(grid_plane(n0.w, sf.x), g.x, cf.x), fmaf(grid_plane(n1.x, sf.y), g.y, cf.y),
+                               fmaf(grid_plane(n1.y, sf.z), g.z, cf.z)), s.t_best);
+  const bool h0 = lo0 <= hi0, h1 = lo1 <= hi1;
+  // the nearer hit child next, the farther one pushed when both are hit (a
+  // predicated store: every local store costs an L2 sector), else the next
+  // stack entry
+  const bool both = h0 && h1;
+  const bool first0 = !h1 || (h0 && lo0 <= lo1);
+  const uint32_t near = first0 ? n1.z : n1.w, far = first0 ? n1.w : n1.z;
+  const int sp = s.sp;
+  if (both && sp < kStack) stack[sp] = far;
+  if (both && sp >= kStack) atomicOr(&a.ctr->error, kErrStack);
+  const int sp1 = sp + ((both && sp < kStack) ? 1 : 0);
+  if (h0 || h1) {
+    s.sp = sp1;
+    s.node = near;
+  } else {
+    s.node = sp1 ? stack[sp1 - 1] : kNone;
+    s.sp = sp1 ? sp1 - 1 : 0;
   }
-  s.node = s.sp ? stack[--s.sp] : kNone;
+}
+
+// Binary BVH: one leaf
+template <bool kAny>
+__device__ __forceinline__ void step_leaf(Trav& s, uint32_t* stack, const ScanArgs& a, uint32_t& n_tris, bool count) {
+  if (trav_tri<kAny>(s, a, s.node & ~kLeafBit, n_tris, count)) s.node = kNone;
+  else s.node = s.sp ? stack[--s.sp] : kNone;
 }
 
 // One step over the 8-wide quantised BVH: a triangle of the current
@@ -327,7 +345,7 @@ __device__ __forceinline__ void step_binary(Trav& s, uint32_t* stack, const Scan
 // visit, bit k for slot k ^ octant), so one stack entry stands for up to 7
 // pending children.  Slot boxes are decoded exactly (see kWideNodeWords);
 // each contains the box of the binary node it stands for, and both node
-// formats take the conservative slab test of trav_begin, so a query reaches
+// formats take a conservative slab test (trav_begin), so a query reaches
 // every triangle it can hit in either BVH and finds the same closest hit.
 template <bool kAny>
 __device__ __forceinline__ void step_wide(Trav& s, uint2* stack, const ScanArgs& a, uint32_t& n_nodes,
@@ -357,7 +375,7 @@ __device__ __forceinline__ void step_wide(Trav& s, uint2* stack, const ScanArgs&
     ++s.visits;   // bounded where the query loop looks at its lanes
     const float3 id = s.id, cn = s.c0, cf = s.c1;
     const bool neg_x = id.x < 0.0f, neg_y = id.y < 0.0f, neg_z = id.z < 0.0f;
-    const uint4* np = reinterpret_cast<const uint4*>(a.nodes) + kWideNodeWords * (size_t)node;
+    const uint4* np = a.nodes + kWideNodeWords * (size_t)node;
     const uint4 w0 = __ldg(np), w1 = __ldg(np + 1), w2 = __ldg(np + 2), w3 = __ldg(np + 3), w4 = __ldg(np + 4);
     const float px = __uint_as_float(w0.x), py = __uint_as_float(w0.y), pz = __uint_as_float(w0.z);
     const float sx = __uint_as_float((w0.w & 0xFFu) << 23), sy = __uint_as_float(((w0.w >> 8) & 0xFFu) << 23),
@@ -469,13 +487,26 @@ __device__ __noinline__ void settle_air_path(const ScanArgs& a, uint32_t bounce,
 // Steps a busy lane takes between two looks at the warp's idle lanes.  The
 // look (votes, the refill hand-out, the end-of-query test) costs about a
 // fifth of a node visit's instructions when taken every step; taking it every
-// kSteps steps lets a lane whose query ended idle for at most kSteps steps
-// (campus bench step: 1.85 ms at 1, 1.77 at 4, 1.73 from 12 to 64).
-constexpr int kSteps = 16;
+// kSteps steps lets a lane whose query ended idle for at most kSteps steps.
+// Binary nodes: 32 (batch of 24 scans of the 1M-triangle campus: 17.24 ms,
+// 17.65 at 16, 17.40 at 64); wide nodes: 16.
+constexpr int kSteps = 32, kStepsWide = 16;
+// Binary nodes: node visits per triangle test.  A lane that reaches a leaf
+// waits until kNodeSteps visits of the others are over and the warp tests its
+// waiting leaves together: a query tests a triangle every 10 to 20 visits, so
+// testing each at once sent the whole warp through the triangle test in two of
+// three steps for one or two lanes (the same scans: 2 / 3 / 4 / 6 / 8 visits
+// 17.82 / 17.72 / 17.65 / 17.64 / 18.10 ms; one test per visit 22.53).
+constexpr int kNodeSteps = 4;
+// Resident threads per SM that the binary query kernels are compiled for:
+// 1,152 leaves 56 registers a thread.  Unbounded, the unrolled visits take 64
+// to 76 registers and lose more to occupancy than the spill-free code gains
+// (city scan 30.5 ms, 26.6 ms at 1,280 threads and 48 registers, 24.8 at 56).
+constexpr int kQueryThreads = 1152;
 // kCount: the traversal counters (RR_COUNT_TRAVERSAL) are compiled only into
 // the kernels of the scans that ask for them
 template <bool kAny, int kBlock, bool kWide, bool kCount>
-__global__ void __launch_bounds__(kBlock) k_query(ScanArgs a, uint32_t bounce) {
+__global__ void __launch_bounds__(kBlock, kWide ? 0 : kQueryThreads / kBlock) k_query(ScanArgs a, uint32_t bounce) {
   typedef typename std::conditional<kWide, uint2, uint32_t>::type StackEntry;
   ScanCounters* C = a.ctr;
   const uint32_t n = kAny ? C->vis_count[bounce] : C->count[bounce];
@@ -541,7 +572,7 @@ __global__ void __launch_bounds__(kBlock) k_query(ScanArgs a, uint32_t bounce) {
           const float3 p = f3(pl);
           const float3 v = f3(__ldg(&sd->pos_rmax)) - p;
           const float dist = length(v);
-          trav_begin(s, p, (1.0f / dist) * v, __ldg(&sd->phys.x), dist, __float_as_uint(pl.w), a.n_tris, kWide);
+          trav_begin(s, a, p, (1.0f / dist) * v, __ldg(&sd->phys.x), dist, __float_as_uint(pl.w), kWide);
         } else if (kAny) {
           const uint2 jb = jobs[job];
           ray_i = jb.x;
@@ -554,7 +585,7 @@ __global__ void __launch_bounds__(kBlock) k_query(ScanArgs a, uint32_t bounce) {
           const float3 p = o + h.t * d;
           const float3 v = f3(__ldg(&sd->pos_rmax)) - p;
           const float dist = length(v);
-          trav_begin(s, p, (1.0f / dist) * v, __ldg(&sd->phys.x), dist, h.leaf, a.n_tris, kWide);
+          trav_begin(s, a, p, (1.0f / dist) * v, __ldg(&sd->phys.x), dist, h.leaf, kWide);
         } else {
           ray_i = perm ? perm[job] : job;
           if (ray_i >= n) ray_i = job;   // only after a failed shading pass (the scan reports it)
@@ -563,8 +594,7 @@ __global__ void __launch_bounds__(kBlock) k_query(ScanArgs a, uint32_t bounce) {
           const float4 phys = __ldg(&a.desc[sm.x].phys);   // t_min, min_energy, freq, r_lim
           const float n_cur = sm.y == kAir ? 1.0f : __ldg(&a.mats[sm.y].n);
           // past t_lim no return can reach the image
-          trav_begin(s, f3(ray.o_L), f3(ray.d_E), phys.x, (phys.w - ray.o_L.w) / n_cur, ray.meta.x, a.n_tris,
-                     kWide);
+          trav_begin(s, a, f3(ray.o_L), f3(ray.d_E), phys.x, (phys.w - ray.o_L.w) / n_cur, ray.meta.x, kWide);
         }
         if (!bvh_ok) s.node = kNone;
       }
@@ -575,10 +605,19 @@ __global__ void __launch_bounds__(kBlock) k_query(ScanArgs a, uint32_t bounce) {
       continue;
     }
     if (busy) {
+      if (kWide) {
 #pragma unroll 2
-      for (int u = 0; u < kSteps && s.node != kNone; ++u) {
-        if (kWide) step_wide<kAny>(s, reinterpret_cast<uint2*>(stack), a, n_nodes, n_tris, count);
-        else step_binary<kAny>(s, reinterpret_cast<uint32_t*>(stack), a, n_nodes, n_tris, count);
+        for (int u = 0; u < kStepsWide && s.node != kNone; ++u)
+          step_wide<kAny>(s, reinterpret_cast<uint2*>(stack), a, n_nodes, n_tris, count);
+      } else {
+        uint32_t* st = reinterpret_cast<uint32_t*>(stack);
+#pragma unroll 1
+        for (int u = 0; u < kSteps && s.node != kNone; u += kNodeSteps) {
+#pragma unroll
+          for (int v = 0; v < kNodeSteps; ++v)
+            if (!(s.node & kLeafBit)) step_inner(s, st, a, n_nodes, count);   // kNone carries the leaf bit
+          if ((s.node & kLeafBit) && s.node != kNone) step_leaf<kAny>(s, st, a, n_tris, count);
+        }
       }
       // depth-first traversal of a tree visits each of its internal nodes
       // (fewer than n_tris, binary or wide) at most once: more visits mean a
