@@ -168,6 +168,11 @@ constexpr uint32_t kSelLo = 0x7104u, kSelHi = 0x7324u, kSelFlip = 0x0220u;
 __device__ __forceinline__ float grid_plane(uint32_t word, uint32_t sel) {
   return __uint_as_float(__byte_perm(word, 0x3F000000u, sel));
 }
+__device__ __forceinline__ float rcp_approx(float x) {
+  float r;
+  asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
 __device__ __forceinline__ float max3(float a, float b, float c) {
   float d;
   asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
@@ -200,16 +205,17 @@ struct Trav {
   uint32_t oct;                               // wide: direction octant
   uint32_t g_base, g_bits;                    // wide: node group
   uint32_t t_base, t_bits;                    // wide: triangles still to test, bit i = triangle t_base + i
-  int sp;
+  int sp;                                     // wide: entries; binary: byte offset of the next free entry
 };
 
 __device__ __forceinline__ void trav_begin(Trav& s, const ScanArgs& a, float3 o, float3 d, float t_min, float t_best,
                                            uint32_t skip, bool wide) {
   s.w = make_woop(o, d);
-  s.id = make_float3(1.0f / (fabsf(d.x) > 1e-30f ? d.x : copysignf(1e-30f, d.x)),
-                     1.0f / (fabsf(d.y) > 1e-30f ? d.y : copysignf(1e-30f, d.y)),
-                     1.0f / (fabsf(d.z) > 1e-30f ? d.z : copysignf(1e-30f, d.z)));
+  const float3 dn = make_float3(fabsf(d.x) > 1e-30f ? d.x : copysignf(1e-30f, d.x),
+                                fabsf(d.y) > 1e-30f ? d.y : copysignf(1e-30f, d.y),
+                                fabsf(d.z) > 1e-30f ? d.z : copysignf(1e-30f, d.z));
   if (wide) {
+    s.id = make_float3(1.0f / dn.x, 1.0f / dn.y, 1.0f / dn.z);
     // Slab test with one fma per plane: plane b is reached at t = fma(b, id, c)
     // with c = -(o id) -+ eps, where the robust form (b - o) id needs two
     // operations.  The fma form errs against (b - o) id by at most u |o id|
@@ -224,12 +230,14 @@ __device__ __forceinline__ void trav_begin(Trav& s, const ScanArgs& a, float3 o,
     s.c1 = make_float3(-ox + ex, -oy + ey, -oz + ez);
   } else {
     // The same over grid planes base + F scale, F in [0.5, 2): t = fma(F, g, c)
-    // with g = scale id and c = (base - o) id.  Against the exact plane
-    // distance the rounded g errs by u |g| per unit of F, c by 3 u |c| and the
-    // fma by u |t|, and |t| <= 2 |g| + |c|: together with the relative
-    // far-plane inflation of the robust slab test (6 u |t|) less than
-    // eps = 24 u (2 |g| + |c|), which moves every near plane down and every
-    // far plane up, so that no inflation is left for the node visits.
+    // with g = scale id and c = (base - o) id, id the hardware's approximate
+    // reciprocal (2 u relative).  Against the exact plane distance the rounded
+    // g errs by 3 u |g| per unit of F, c by 4 u |c| and the fma by u |t|, and
+    // |t| <= 2 |g| + |c|: together with the relative far-plane inflation of
+    // the robust slab test (6 u |t|) less than eps = 24 u (2 |g| + |c|), which
+    // moves every near plane down and every far plane up, so that no
+    // inflation is left for the node visits.
+    s.id = make_float3(rcp_approx(dn.x), rcp_approx(dn.y), rcp_approx(dn.z));
     const float4 base = __ldg(a.frame), scale = __ldg(a.frame + 1);
     const float cx = __fmul_rn(base.x - o.x, s.id.x), cy = __fmul_rn(base.y - o.y, s.id.y),
                 cz = __fmul_rn(base.z - o.z, s.id.z);
@@ -248,7 +256,7 @@ __device__ __forceinline__ void trav_begin(Trav& s, const ScanArgs& a, float3 o,
   s.best = kNone;
   s.best_id = 0u;
   s.visits = 0u;
-  s.sp = 0;
+  s.sp = wide ? 0 : 4;   // binary: above the kNone entry
   if (wide) {
     s.oct = (s.id.x < 0.0f ? 1u : 0u) | (s.id.y < 0.0f ? 2u : 0u) | (s.id.z < 0.0f ? 4u : 0u);
     s.g_base = 0u;
@@ -287,6 +295,11 @@ __device__ __forceinline__ bool trav_tri(Trav& s, const ScanArgs& a, uint32_t j,
   return false;
 }
 
+// Stack entry at byte offset sp of a binary traversal
+__device__ __forceinline__ uint32_t& bin_entry(uint32_t* stack, int sp) {
+  return *reinterpret_cast<uint32_t*>(reinterpret_cast<char*>(stack) + sp);
+}
+
 // Binary BVH: one inner node (both children tested, nearer first).
 __device__ __forceinline__ void step_inner(Trav& s, uint32_t* stack, const ScanArgs& a, uint32_t& n_nodes,
                                            bool count) {
@@ -310,28 +323,30 @@ __device__ __forceinline__ void step_inner(Trav& s, uint32_t* stack, const ScanA
   const bool h0 = lo0 <= hi0, h1 = lo1 <= hi1;
   // the nearer hit child next, the farther one pushed when both are hit (a
   // predicated store: every local store costs an L2 sector), else the next
-  // stack entry
+  // stack entry.  The lowest entry is kNone, so popping it ends the query
+  // without a test, and a full stack is noticed by the query loop, not here.
   const bool both = h0 && h1;
   const bool first0 = !h1 || (h0 && lo0 <= lo1);
   const uint32_t near = first0 ? n1.z : n1.w, far = first0 ? n1.w : n1.z;
-  const int sp = s.sp;
-  if (both && sp < kStack) stack[sp] = far;
-  if (both && sp >= kStack) atomicOr(&a.ctr->error, kErrStack);
-  const int sp1 = sp + ((both && sp < kStack) ? 1 : 0);
+  if (both) bin_entry(stack, s.sp) = far;
+  s.sp += both ? 4 : 0;   // apart from the store: a branch over both costs 5-7 % of a scan
   if (h0 || h1) {
-    s.sp = sp1;
     s.node = near;
   } else {
-    s.node = sp1 ? stack[sp1 - 1] : kNone;
-    s.sp = sp1 ? sp1 - 1 : 0;
+    s.sp -= 4;
+    s.node = bin_entry(stack, s.sp);
   }
 }
 
 // Binary BVH: one leaf
 template <bool kAny>
 __device__ __forceinline__ void step_leaf(Trav& s, uint32_t* stack, const ScanArgs& a, uint32_t& n_tris, bool count) {
-  if (trav_tri<kAny>(s, a, s.node & ~kLeafBit, n_tris, count)) s.node = kNone;
-  else s.node = s.sp ? stack[--s.sp] : kNone;
+  if (trav_tri<kAny>(s, a, s.node & ~kLeafBit, n_tris, count)) {
+    s.node = kNone;
+  } else {
+    s.sp -= 4;
+    s.node = bin_entry(stack, s.sp);
+  }
 }
 
 // One step over the 8-wide quantised BVH: a triangle of the current
@@ -498,6 +513,11 @@ constexpr int kSteps = 32, kStepsWide = 16;
 // three steps for one or two lanes (the same scans: 2 / 3 / 4 / 6 / 8 visits
 // 17.82 / 17.72 / 17.65 / 17.64 / 18.10 ms; one test per visit 22.53).
 constexpr int kNodeSteps = 4;
+// Binary stack: kNone, kStack entries, and room for the pushes of one group of
+// kNodeSteps visits, after which the query loop checks the depth.  The check
+// at every push and pop, with the divisions of trav_begin, was 6 % of a scan
+// (campus scan 1,134 -> 1,061 us, city scan 24.9 -> 23.4 ms).
+constexpr int kBinStack = 1 + kStack + kNodeSteps;
 // Resident threads per SM that the binary query kernels are compiled for:
 // 1,152 leaves 56 registers a thread.  Unbounded, the unrolled visits take 64
 // to 76 registers and lose more to occupancy than the spill-free code gains
@@ -532,7 +552,7 @@ __global__ void __launch_bounds__(kBlock, kWide ? 0 : kQueryThreads / kBlock) k_
   const uint32_t refill = a.refill;
   Trav s;
   s.node = kNone;
-  StackEntry stack[kStack];
+  StackEntry stack[kWide ? kStack : kBinStack];
   uint32_t ray_i = kNone;   // ray of the lane's query (kNone: idle)
   float wa = 0.0f;          // any hit: W(omega_a) of the candidate
   uint32_t c_base = 0u, c_end = 0u;   // claimed, unassigned jobs (warp-uniform)
@@ -596,6 +616,7 @@ __global__ void __launch_bounds__(kBlock, kWide ? 0 : kQueryThreads / kBlock) k_
           // past t_lim no return can reach the image
           trav_begin(s, a, f3(ray.o_L), f3(ray.d_E), phys.x, (phys.w - ray.o_L.w) / n_cur, ray.meta.x, kWide);
         }
+        if (!kWide) bin_entry(reinterpret_cast<uint32_t*>(stack), 0) = kNone;
         if (!bvh_ok) s.node = kNone;
       }
     }
@@ -617,6 +638,11 @@ __global__ void __launch_bounds__(kBlock, kWide ? 0 : kQueryThreads / kBlock) k_
           for (int v = 0; v < kNodeSteps; ++v)
             if (!(s.node & kLeafBit)) step_inner(s, st, a, n_nodes, count);   // kNone carries the leaf bit
           if ((s.node & kLeafBit) && s.node != kNone) step_leaf<kAny>(s, st, a, n_tris, count);
+          if (s.sp > 4 * (1 + kStack)) {   // a tree deeper than the stack: the scan reports it
+            atomicOr(&a.ctr->error, kErrStack);
+            s.node = kNone;
+            s.sp = 0;
+          }
         }
       }
       // depth-first traversal of a tree visits each of its internal nodes
