@@ -26,7 +26,7 @@
 
 namespace rr {
 
-constexpr int kImgBlock = 256;
+constexpr int kImgBlock = 256;       // beam pattern pass
 constexpr int kMaxTaps = 2 * 768 + 1;   // blur / pattern radius up to 768
 
 __device__ __forceinline__ int gauss_taps(float sigma, float* w) {
@@ -115,7 +115,10 @@ __device__ __forceinline__ void bin_add(unsigned long long* cell, float x, float
   } while (old != seen);
 }
 
-__global__ void __launch_bounds__(kImgBlock) k_bin_column(ScanArgs a) {
+// A column is one block's work: with few columns the chip is filled by wider
+// blocks (launch_image).
+template <int kBlock>
+__global__ void __launch_bounds__(kBlock) k_bin_column(ScanArgs a) {
   extern __shared__ unsigned long long sm64[];
   unsigned long long* cells = sm64;                             // [n_bins] (sum, correction)
   float* hist = reinterpret_cast<float*>(sm64 + a.max_bins);    // [n_bins] the compensated sums
@@ -298,14 +301,18 @@ static size_t bin_smem(uint32_t n_bins) { return (size_t)n_bins * (sizeof(unsign
 void init_image_attrs() {
   static bool attr_set = false;
   if (!attr_set) {
-    cudaFuncSetAttribute(k_bin_column, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bin_smem(RR_MAX_BINS));
+    for (const void* k : {(const void*)k_bin_column<256>, (const void*)k_bin_column<512>, (const void*)k_bin_column<1024>})
+      cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bin_smem(RR_MAX_BINS));
     attr_set = true;
   }
 }
 
 cudaError_t launch_image(const ScanArgs& a, bool pattern, cudaStream_t st) {
   init_image_attrs();
-  k_bin_column<<<a.n_cols, kImgBlock, bin_smem(a.max_bins), st>>>(a);
+  const uint32_t sms = (uint32_t)num_sms();
+  if (a.n_cols <= 2u * sms) k_bin_column<1024><<<a.n_cols, 1024, bin_smem(a.max_bins), st>>>(a);
+  else if (a.n_cols <= 4u * sms) k_bin_column<512><<<a.n_cols, 512, bin_smem(a.max_bins), st>>>(a);
+  else k_bin_column<256><<<a.n_cols, 256, bin_smem(a.max_bins), st>>>(a);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   if (pattern) {
@@ -345,6 +352,18 @@ cudaError_t launch_db_u8(const float* polar, uint64_t n, float cutoff_db, uint8_
 
 using namespace rr_host;
 
+// device memory of the current device that a kernel can take as 4-byte elements
+static bool usable_here(const void* p) {
+  cudaPointerAttributes at;
+  int dev = -1;
+  if (reinterpret_cast<uintptr_t>(p) % 4 != 0 || cudaGetDevice(&dev) != cudaSuccess ||
+      cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return at.type == cudaMemoryTypeDevice && at.device == dev;
+}
+
 extern "C" int rr_accumulate_returns(const uint32_t* column, const uint32_t* bin, const float* energy, uint64_t n,
                                      uint32_t n_columns, uint32_t n_bins, float* out) {
   if (!out || (n && (!column || !bin || !energy))) return fail(RR_ERR_INVALID_ARG, "NULL buffer");
@@ -353,54 +372,66 @@ extern "C" int rr_accumulate_returns(const uint32_t* column, const uint32_t* bin
   if (n >= (1ull << 31)) return fail(RR_ERR_INVALID_ARG, "at most 2^31 - 1 returns");
   cudaStream_t st = current_stream();
   const size_t img_bytes = (size_t)n_columns * n_bins * sizeof(float);
-  // device scratch of this call: inputs, records, a counter block, one scan
-  // descriptor with its prefix arrays, the image
-  uint32_t *d_col = nullptr, *d_bin = nullptr, *d_bad = nullptr;
-  float *d_e = nullptr, *d_img = nullptr;
-  uint2* d_recs = nullptr;
-  ScanCounters* d_ctr = nullptr;
-  ScanDesc* d_desc = nullptr;
-  uint32_t* d_pre = nullptr;
+  // Buffers of this device are read and written where they are; others (host
+  // memory, another device's, or not aligned to their elements) go through
+  // the scratch of this call, one allocation: [column][bin][energy][records]
+  // [image][setup].  Nine allocations and the copies of device inputs were
+  // most of a call.
+  const bool own_col = usable_here(column), own_bin = usable_here(bin), own_e = usable_here(energy),
+             own_out = usable_here(out);
+  const size_t nn = n ? n : 1;
+  struct Setup {
+    ScanCounters ctr;
+    ScanDesc desc;
+    uint32_t pre[4], bad;   // ray prefix (unused) and column prefix; the check's flag
+  };
+  auto up = [](size_t x) { return (x + 255) & ~size_t(255); };
+  const size_t in_bytes = up(nn * 4);
+  size_t off = 0, o_col = 0, o_bin = 0, o_e = 0, o_img = 0;
+  if (!own_col) o_col = off, off += in_bytes;
+  if (!own_bin) o_bin = off, off += in_bytes;
+  if (!own_e) o_e = off, off += in_bytes;
+  const size_t o_recs = off;
+  off += up(nn * 8);
+  if (!own_out) o_img = off, off += up(img_bytes);
+  const size_t o_setup = off;
+  off += up(sizeof(Setup));
+  char* w = nullptr;
+  cudaError_t e = dev_malloc(&w, off);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return cuda_fail(e, "accumulating the returns");
+  }
   auto cleanup = [&]() {
     cudaStreamSynchronize(st);
-    for (void* p : {(void*)d_col, (void*)d_bin, (void*)d_bad, (void*)d_e, (void*)d_img, (void*)d_recs, (void*)d_ctr,
-                    (void*)d_desc, (void*)d_pre})
-      if (p) cudaFree(p);
+    cudaFree(w);
   };
-  cudaError_t e = cudaSuccess;
-  const size_t nn = n ? n : 1;
-  if (e == cudaSuccess) e = dev_malloc(&d_col, nn * 4);
-  if (e == cudaSuccess) e = dev_malloc(&d_bin, nn * 4);
-  if (e == cudaSuccess) e = dev_malloc(&d_e, nn * 4);
-  if (e == cudaSuccess) e = dev_malloc(&d_recs, nn * 8);
-  if (e == cudaSuccess) e = dev_malloc(&d_bad, 4);
-  if (e == cudaSuccess) e = dev_malloc(&d_img, img_bytes);
-  if (e == cudaSuccess) e = dev_malloc(&d_ctr, sizeof(ScanCounters));
-  if (e == cudaSuccess) e = dev_malloc(&d_desc, sizeof(ScanDesc));
-  if (e == cudaSuccess) e = dev_malloc(&d_pre, 4 * sizeof(uint32_t));
-  if (e == cudaSuccess && n) e = cudaMemcpyAsync(d_col, column, n * 4, cudaMemcpyDefault, st);
-  if (e == cudaSuccess && n) e = cudaMemcpyAsync(d_bin, bin, n * 4, cudaMemcpyDefault, st);
-  if (e == cudaSuccess && n) e = cudaMemcpyAsync(d_e, energy, n * 4, cudaMemcpyDefault, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(d_bad, 0, 4, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(d_ctr, 0, sizeof(ScanCounters), st);
-  ScanDesc desc;
-  memset(&desc, 0, sizeof desc);
-  desc.dims = make_uint4(n_columns, 1u, 1u, n_bins);
-  desc.offs = make_uint4(0u, 0u, kNone, 0u);
-  desc.image = d_img;
-  const uint32_t pre[4] = {0u, 0u, 0u, n_columns};   // ray prefix (unused) and column prefix
-  const uint32_t starts[2] = {0u, (uint32_t)n};
-  if (e == cudaSuccess) e = cudaMemcpyAsync(d_desc, &desc, sizeof desc, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(d_pre, pre, sizeof pre, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&d_ctr->rec_start[0], starts, sizeof starts, cudaMemcpyHostToDevice, st);
+  const uint32_t* d_col = own_col ? column : (const uint32_t*)(w + o_col);
+  const uint32_t* d_bin = own_bin ? bin : (const uint32_t*)(w + o_bin);
+  const float* d_e = own_e ? energy : (const float*)(w + o_e);
+  uint2* d_recs = (uint2*)(w + o_recs);
+  float* d_img = own_out ? out : (float*)(w + o_img);
+  Setup* d_setup = (Setup*)(w + o_setup);
+  if (n && !own_col) e = cudaMemcpyAsync(w + o_col, column, n * 4, cudaMemcpyDefault, st);
+  if (e == cudaSuccess && n && !own_bin) e = cudaMemcpyAsync(w + o_bin, bin, n * 4, cudaMemcpyDefault, st);
+  if (e == cudaSuccess && n && !own_e) e = cudaMemcpyAsync(w + o_e, energy, n * 4, cudaMemcpyDefault, st);
+  Setup setup;
+  memset(&setup, 0, sizeof setup);
+  setup.desc.dims = make_uint4(n_columns, 1u, 1u, n_bins);
+  setup.desc.offs = make_uint4(0u, 0u, kNone, 0u);
+  setup.desc.image = d_img;
+  setup.pre[3] = n_columns;
+  setup.ctr.rec_start[1] = (uint32_t)n;
+  if (e == cudaSuccess) e = cudaMemcpyAsync(d_setup, &setup, sizeof setup, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess && n) {
     k_pack_returns<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(d_col, d_bin, d_e, (uint32_t)n, n_columns, n_bins,
-                                                                 d_recs, d_bad);
+                                                                 d_recs, &d_setup->bad);
     e = cudaGetLastError();
   }
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st);   // the host copies above came from the stack
+  // the check's answer before anything is written to the output
   uint32_t bad = 0;
-  if (e == cudaSuccess) e = cudaMemcpy(&bad, d_bad, 4, cudaMemcpyDeviceToHost);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(&bad, &d_setup->bad, 4, cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) {
     cudaGetLastError();
     cleanup();
@@ -412,24 +443,24 @@ extern "C" int rr_accumulate_returns(const uint32_t* column, const uint32_t* bin
   }
   ScanArgs a;
   memset(&a, 0, sizeof a);
-  a.desc = d_desc;
-  a.ray0 = d_pre;
-  a.col0 = d_pre + 2;
+  a.desc = &d_setup->desc;
+  a.ray0 = d_setup->pre;
+  a.col0 = d_setup->pre + 2;
   a.n_scans = 1;
   a.n_cols = n_columns;
   a.max_bounces = 1;
   a.max_bins = n_bins;
   a.recs = d_recs;
-  a.ctr = d_ctr;
+  a.ctr = &d_setup->ctr;
   a.rec_cap = (uint32_t)nn;
   e = launch_image(a, false, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(out, d_img, img_bytes, cudaMemcpyDefault, st);
+  if (e == cudaSuccess && !own_out) e = cudaMemcpyAsync(out, d_img, img_bytes, cudaMemcpyDefault, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) {
     cudaGetLastError();
     cleanup();
     return cuda_fail(e, "accumulating the returns");
   }
-  cleanup();
+  cudaFree(w);
   return RR_OK;
 }
