@@ -392,7 +392,8 @@ int rr_scan_batch_async(rr_scene* scene, uint32_t n, const rr_pose* poses, const
                         azimuth ranges, each on its own stream, so that the
                         slow queries closing one range's bounce overlap the
                         other ranges' work (1..4; 0: the default, 3).  Scans
-                        with a beam pattern run whole.  The image is the same
+                        with a beam pattern run whole, and while the value is
+                        the default so do scans too small to gain from it.  The image is the same
                         up to the rounding of the bin sums.
    bvh_build            RR_BVH_SAH_TOP (default): the LBVH (Morton codes,
                         radix sort, Karras hierarchy, refit) with the part

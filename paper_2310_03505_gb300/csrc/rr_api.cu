@@ -210,10 +210,15 @@ int check_device(const rr_scene* s, const char* who) {
   return RR_OK;
 }
 
-// read (and clear) the sticky device status of a context; waits for the stream
-int device_status(ExecCtx* x, cudaStream_t st) {
+// Read (and clear) the sticky device status of a context in two halves, so
+// that the contexts of a split scan are read side by side.
+static int status_request(ExecCtx* x, cudaStream_t st) {
   RR_CHECK_CUDA(cudaMemcpyAsync(x->h_ctr, x->d_ctr, sizeof(ScanCounters), cudaMemcpyDeviceToHost, st),
                 "reading the scan counters");
+  return RR_OK;
+}
+
+static int status_wait(ExecCtx* x, cudaStream_t st) {
   RR_CHECK_CUDA(cudaStreamSynchronize(st), "scan");
   const uint32_t err = x->h_ctr->error;
   if (err) {
@@ -239,10 +244,22 @@ int device_status(ExecCtx* x, cudaStream_t st) {
   return RR_OK;
 }
 
+// waits for the stream
+int device_status(ExecCtx* x, cudaStream_t st) {
+  const int rc = status_request(x, st);
+  return rc == RR_OK ? status_wait(x, st) : rc;
+}
+
 int scene_status(rr_scene* s, cudaStream_t st) {
-  int rc = device_status(&s->main, st);   // st has joined the split lanes' work
+  int rc = status_request(&s->main, st);   // st has joined the split lanes' work
   for (uint32_t k = 0; k < s->split_used; ++k) {
-    const int r = device_status(&s->split[k].ctx, s->split[k].stream);
+    const int r = status_request(&s->split[k].ctx, s->split[k].stream);
+    if (rc == RR_OK) rc = r;
+  }
+  if (rc != RR_OK) return rc;
+  rc = status_wait(&s->main, st);
+  for (uint32_t k = 0; k < s->split_used; ++k) {
+    const int r = status_wait(&s->split[k].ctx, s->split[k].stream);
     if (rc == RR_OK) rc = r;
   }
   return rc;

@@ -531,6 +531,18 @@ int batch_run(rr_scene* s, ExecCtx* x, const rr_pose* poses, const rr_sensor_par
   return RR_OK;
 }
 
+// Whether a scan runs whole although the default would split it.  The ranges
+// overlap each other's slow queries, which pays once a bounce lasts well
+// beyond its launches: with few rays, or in a scene of few triangles (short
+// queries), the extra launches and the joins cost more.  Measured, split in 3
+// against whole: tiny room 3,200 rays 217 / 183 us and 40,000 rays 320 / 277;
+// 200k-triangle campus 12,000 rays 596 / 550, 24,000 rays 669 / 693, 40,000
+// rays 789 / 868; 5M-triangle city 24,000 rays 1,119 / 1,251.
+static bool scan_whole(const rr_scene* s, const rr_sensor_params* p) {
+  const uint64_t rays = (uint64_t)p->n_azimuth * p->rays_per_beam;
+  return rays < (1u << 14) || (s->nt < (1u << 13) && rays < (1u << 16));
+}
+
 // One scan as split_streams azimuth ranges, each a launch sequence of its own
 // on its own stream and execution context: the bounces of the ranges no
 // longer wait for each other, so the tail of one range's bounce (its slowest
@@ -539,6 +551,7 @@ int batch_run(rr_scene* s, ExecCtx* x, const rr_pose* poses, const rr_sensor_par
 int scan_split(rr_scene* s, const rr_pose* pose, const rr_sensor_params* p, float* image, cudaStream_t st,
                bool profile) {
   uint32_t k_n = std::min<uint32_t>(s->cfg.split, p->n_azimuth);
+  if (s->cfg.split_auto && scan_whole(s, p)) k_n = 1;
   if (k_n <= 1 || p->az_pattern_sigma > 0.f) {
     float* const images[1] = {image};
     return batch_run(s, &s->main, pose, p, images, 1, nullptr, st, s->cfg);
@@ -715,7 +728,10 @@ int rr_batch_config_set(rr_scene* s, const rr_batch_config* c) {
   const int rc = cfg_check(c);
   if (rc != RR_OK) return rc;
   const bool rebuild = c->bvh_build != s->cfg.bvh_build;
+  // a split_streams that was not changed from the default stays a default
+  const bool split_auto = c->split_streams == 0 || (s->cfg.split_auto && c->split_streams == s->cfg.split);
   s->cfg = cfg_from_abi(c);
+  s->cfg.split_auto = split_auto;
   return rebuild ? rebuild_bvh(s, current_stream()) : RR_OK;
 }
 

@@ -31,6 +31,7 @@ struct LaunchCfg {
   uint32_t node_format = RR_NODES_BINARY;
   uint32_t refill = 16;               // idle lanes that trigger a refill (1..32)
   uint32_t split = 3;                 // a single scan as this many azimuth ranges on their own streams
+  bool split_auto = true;             // split is the library's default: small scans run whole (scan_whole)
   uint64_t ws_limit = uint64_t(24) << 30;
   uint32_t bvh_build = RR_BVH_SAH_TOP;
   uint32_t order = 0;                 // RR_ORDER_*: query order of the closest-hit queries of bounces >= 1
