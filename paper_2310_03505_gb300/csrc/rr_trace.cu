@@ -29,7 +29,6 @@
 namespace rr {
 
 constexpr int kShadeBlock = 256;
-constexpr float kBoxInflate = 1.00000036f;  // 1 + 2 gamma_3 (robust slab test, Ize 2013): wide nodes
 
 // ---------------------------------------------------------------------------
 // beam axis angle 2 pi a / n with an exact quadrant reduction; returns (cos, sin)
@@ -204,8 +203,8 @@ struct Trav {
   uint32_t best, best_id, visits;
   uint32_t oct;                               // wide: direction octant
   uint32_t g_base, g_bits;                    // wide: node group
-  uint32_t t_base, t_bits;                    // wide: triangles still to test, bit i = triangle t_base + i
-  int sp;                                     // wide: entries; binary: byte offset of the next free entry
+  uint32_t t_base, t_bits, t_counts;          // wide: a node's first triangle, hit leaf slots still to test, slot counts
+  int sp;                                     // next free stack entry (binary: its byte offset)
 };
 
 __device__ __forceinline__ void trav_begin(Trav& s, const ScanArgs& a, float3 o, float3 d, float t_min, float t_best,
@@ -222,8 +221,9 @@ __device__ __forceinline__ void trav_begin(Trav& s, const ScanArgs& a, float3 o,
     // (o id rounded) + u |c| (c rounded) + u |t| (the fma itself), u = 2^-24.
     // eps = 4 u |o id| moves every near plane down and every far plane up by
     // more than the first two; the last is relative, like the errors of the
-    // robust form, and the far-plane inflation kBoxInflate covers it.  So a box
-    // the robust test accepts is accepted here too.
+    // robust form, and is covered with the far-plane inflation of the robust
+    // slab test (1 + 2 gamma_3, Ize 2013) at the node.  So a box the robust
+    // test accepts is accepted here too.
     const float ox = __fmul_rn(o.x, s.id.x), oy = __fmul_rn(o.y, s.id.y), oz = __fmul_rn(o.z, s.id.z);
     const float ex = 0x1p-22f * fabsf(ox), ey = 0x1p-22f * fabsf(oy), ez = 0x1p-22f * fabsf(oz);
     s.c0 = make_float3(-ox - ex, -oy - ey, -oz - ez);
@@ -256,13 +256,14 @@ __device__ __forceinline__ void trav_begin(Trav& s, const ScanArgs& a, float3 o,
   s.best = kNone;
   s.best_id = 0u;
   s.visits = 0u;
-  s.sp = wide ? 0 : 4;   // binary: above the kNone entry
+  s.sp = wide ? 1 : 4;   // above the lowest entry, which ends the query
   if (wide) {
     s.oct = (s.id.x < 0.0f ? 1u : 0u) | (s.id.y < 0.0f ? 2u : 0u) | (s.id.z < 0.0f ? 4u : 0u);
     s.g_base = 0u;
     s.g_bits = (1u << 8) | (1u << s.oct);   // the root: internal slot 0 of a virtual group
     s.t_base = 0u;
     s.t_bits = 0u;
+    s.t_counts = 0u;
     s.node = a.n_tris ? 0u : kNone;
   } else {
     s.node = a.n_tris == 0 ? kNone : (a.n_tris == 1 ? kLeafBit : 0u);
@@ -350,95 +351,115 @@ __device__ __forceinline__ void step_leaf(Trav& s, uint32_t* stack, const ScanAr
   }
 }
 
-// One step over the 8-wide quantised BVH: a triangle of the current
-// triangle group, else the next child of the current node group, else a
-// group from the stack.  A leaf slot holds 1..3 consecutive triangles (its
-// count in two bits of the node's word w1.w); the hit leaf slots of a node
-// become one mask over its up to 24 triangles.  Children are visited in slot order k ^ octant
-// (near first) through node groups as in Ylitie, Karras, Laine, "Efficient
-// incoherent ray traversal on GPUs through compressed wide BVHs" (HPG 2017):
-// a group is (first child, internal-slot mask << 8 | hit children still to
-// visit, bit k for slot k ^ octant), so one stack entry stands for up to 7
-// pending children.  Slot boxes are decoded exactly (see kWideNodeWords);
-// each contains the box of the binary node it stands for, and both node
-// formats take a conservative slab test (trav_begin), so a query reaches
-// every triangle it can hit in either BVH and finds the same closest hit.
+// The 8-wide quantised BVH.  A node visit takes the next child of the current
+// node group, else of a group from the stack; the triangles of the leaf slots
+// it hits are tested before the query visits another node.  A leaf slot holds
+// 1..3 consecutive triangles (its count in two bits of the node's word w1.w).
+// Children are visited in slot order k ^ octant (near first) through node
+// groups as in Ylitie, Karras, Laine, "Efficient incoherent ray traversal on
+// GPUs through compressed wide BVHs" (HPG 2017): a group is (first child,
+// internal-slot mask << 8 | hit children still to visit, bit k for slot
+// k ^ octant), so one stack entry stands for up to 7 pending children; the
+// lowest entry is empty and ends the query.  Slot boxes (see kWideNodeWords)
+// contain the box of the binary node they stand for, and both node formats
+// take a conservative slab test, so a query reaches every triangle it can hit
+// in either BVH and finds the same closest hit.
+//
+// Slab test: byte q of a plane word becomes the float F = 1 + q 2^-15 (bits
+// 0x3F80qq00), and the plane P + q s is reached at t = fma(F, g, c) with
+// g = 2^15 s id and c = (P - 2^15 s) id - o id: one fma a plane where decoding
+// the plane first took two.  P - 2^15 s is exact; the roundings of g, c and
+// the fma err by less than 2^-23 (2 |g| + |c|), the far-plane inflation of the
+// robust test (6 u |t|) by less than 2^-21 of it, and e = 2^-20 (|g| + |c|),
+// 1/32 of a quantum and more, covers both: it moves near planes down and far
+// planes up.
+//
+// The former step took a triangle, a node or a stack entry, whichever was
+// next, so a warp ran all three for a few lanes each, decoded every plane
+// before its slab fma and set the hit masks slot by slot behind branches:
+// campus scan over the wide nodes 2,447 us, 1,567 now (batch server's burst of
+// 24 requests 18.3 -> 12.1 ms); 1 / 3 visits per leaf test 1,590 / 1,658.
 template <bool kAny>
-__device__ __forceinline__ void step_wide(Trav& s, uint2* stack, const ScanArgs& a, uint32_t& n_nodes,
-                                          uint32_t& n_tris, bool count) {
-  const uint32_t oct = s.oct;
-  if (s.t_bits) {
-    const uint32_t j = s.t_base + (uint32_t)__ffs(s.t_bits) - 1u;
-    s.t_bits &= s.t_bits - 1u;
-    if (j < a.n_tris && trav_tri<kAny>(s, a, j, n_tris, count)) s.node = kNone;
-    return;
-  }
-  if (s.g_bits & 0xFFu) {
-    const uint32_t k = __ffs(s.g_bits & 0xFFu) - 1u;
-    s.g_bits &= ~(1u << k);
-    const uint32_t slot = k ^ oct;
-    const uint32_t node = s.g_base + __popc((s.g_bits >> 8) & ((1u << slot) - 1u));
-    if (s.g_bits & 0xFFu) {
-      if (s.sp < kStack) stack[s.sp++] = make_uint2(s.g_base, s.g_bits);
-      else atomicOr(&a.ctr->error, kErrStack);
-    }
-    if (node >= a.node_cap) {   // only a failed build can get here
-      atomicOr(&a.ctr->error, kErrBvh);
-      s.node = kNone;
-      return;
-    }
-    if (count) ++n_nodes;
-    ++s.visits;   // bounded where the query loop looks at its lanes
-    const float3 id = s.id, cn = s.c0, cf = s.c1;
-    const bool neg_x = id.x < 0.0f, neg_y = id.y < 0.0f, neg_z = id.z < 0.0f;
-    const uint4* np = a.nodes + kWideNodeWords * (size_t)node;
-    const uint4 w0 = __ldg(np), w1 = __ldg(np + 1), w2 = __ldg(np + 2), w3 = __ldg(np + 3), w4 = __ldg(np + 4);
-    const float px = __uint_as_float(w0.x), py = __uint_as_float(w0.y), pz = __uint_as_float(w0.z);
-    const float sx = __uint_as_float((w0.w & 0xFFu) << 23), sy = __uint_as_float(((w0.w >> 8) & 0xFFu) << 23),
-                sz = __uint_as_float(((w0.w >> 16) & 0xFFu) << 23);
-    const uint32_t imask = w0.w >> 24, valid = w1.z, counts = w1.w;
-    // near and far plane bytes per axis: (lo, hi) for a positive direction, swapped otherwise
-    const uint32_t nx0 = neg_x ? w3.z : w2.x, nx1 = neg_x ? w3.w : w2.y;
-    const uint32_t fx0 = neg_x ? w2.x : w3.z, fx1 = neg_x ? w2.y : w3.w;
-    const uint32_t ny0 = neg_y ? w4.x : w2.z, ny1 = neg_y ? w4.y : w2.w;
-    const uint32_t fy0 = neg_y ? w2.z : w4.x, fy1 = neg_y ? w2.w : w4.y;
-    const uint32_t nz0 = neg_z ? w4.z : w3.x, nz1 = neg_z ? w4.w : w3.y;
-    const uint32_t fz0 = neg_z ? w3.x : w4.z, fz1 = neg_z ? w3.y : w4.w;
-    uint32_t hit_i = 0u, tmask = 0u, first = 0u;   // first: the slot's first triangle (of the node's)
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      // bits 0x4B0000qq = 2^23 + q (byte q of the word), decoded to P + q s exactly
-      const uint32_t sel = 0x7440u | (uint32_t)(j & 3);
-      const float bnx = fmaf(__uint_as_float(__byte_perm(j < 4 ? nx0 : nx1, 0x4B000000u, sel)), sx, px);
-      const float bfx = fmaf(__uint_as_float(__byte_perm(j < 4 ? fx0 : fx1, 0x4B000000u, sel)), sx, px);
-      const float bny = fmaf(__uint_as_float(__byte_perm(j < 4 ? ny0 : ny1, 0x4B000000u, sel)), sy, py);
-      const float bfy = fmaf(__uint_as_float(__byte_perm(j < 4 ? fy0 : fy1, 0x4B000000u, sel)), sy, py);
-      const float bnz = fmaf(__uint_as_float(__byte_perm(j < 4 ? nz0 : nz1, 0x4B000000u, sel)), sz, pz);
-      const float bfz = fmaf(__uint_as_float(__byte_perm(j < 4 ? fz0 : fz1, 0x4B000000u, sel)), sz, pz);
-      const float lo =
-          fmaxf(fmaxf(fmaf(bnx, id.x, cn.x), fmaf(bny, id.y, cn.y)), fmaxf(fmaf(bnz, id.z, cn.z), s.t_min));
-      const float hi = fminf(
-          fminf(fminf(fmaf(bfx, id.x, cf.x), fmaf(bfy, id.y, cf.y)), fmaf(bfz, id.z, cf.z)) * kBoxInflate, s.t_best);
-      const uint32_t c = counts >> (2 * j) & 3u;   // triangles of a leaf slot (0: inner or empty)
-      if (lo <= hi && (valid >> j & 1u)) {
-        if (imask >> j & 1u) hit_i |= 1u << (j ^ oct);
-        else tmask |= ((1u << c) - 1u) << first;
-      }
-      first += c;
-    }
-    s.g_base = w1.x;
-    s.g_bits = (imask << 8) | hit_i;
-    s.t_base = w1.y;
-    s.t_bits = tmask;
-    return;
-  }
-  if (s.sp) {
-    const uint2 e = stack[--s.sp];
-    s.g_base = e.x;
-    s.g_bits = e.y;
-  } else {
+__device__ __forceinline__ void step_wide_node(Trav& s, uint2* stack, const ScanArgs& a, uint32_t& n_nodes,
+                                               bool count) {
+  const uint2 top = stack[s.sp - 1];
+  const bool pop = !(s.g_bits & 0xFFu);
+  const uint32_t base = pop ? top.x : s.g_base;
+  uint32_t bits = pop ? top.y : s.g_bits;
+  s.sp -= pop ? 1 : 0;
+  if (!(bits & 0xFFu)) {   // the empty entry
     s.node = kNone;
+    return;
   }
+  const uint32_t oct = s.oct, slot = (__ffs(bits) - 1u) ^ oct;
+  bits &= bits - 1u;   // the lowest bit is a pending child's
+  const uint32_t node = min(base + __popc((bits >> 8) & ((1u << slot) - 1u)), a.node_cap - 1u);
+  if (bits & 0xFFu) stack[s.sp] = make_uint2(base, bits);
+  s.sp += (bits & 0xFFu) ? 1 : 0;
+  if (count) ++n_nodes;
+  ++s.visits;   // bounded where the query loop looks at its lanes
+  const float3 id = s.id;
+  const bool neg_x = id.x < 0.0f, neg_y = id.y < 0.0f, neg_z = id.z < 0.0f;
+  const uint4* np = a.nodes + kWideNodeWords * (size_t)node;
+  const uint4 w0 = __ldg(np), w1 = __ldg(np + 1), w2 = __ldg(np + 2), w3 = __ldg(np + 3), w4 = __ldg(np + 4);
+  const float sx = __uint_as_float((w0.w & 0xFFu) << 23), sy = __uint_as_float(((w0.w >> 8) & 0xFFu) << 23),
+              sz = __uint_as_float(((w0.w >> 16) & 0xFFu) << 23);
+  // the node holds P - 2^23 s
+  const float px = fmaf(sx, 8355840.0f, __uint_as_float(w0.x)), py = fmaf(sy, 8355840.0f, __uint_as_float(w0.y)),
+              pz = fmaf(sz, 8355840.0f, __uint_as_float(w0.z));
+  const float3 g = make_float3(32768.0f * sx * id.x, 32768.0f * sy * id.y, 32768.0f * sz * id.z);
+  float3 cn = make_float3(fmaf(px, id.x, s.c0.x), fmaf(py, id.y, s.c0.y), fmaf(pz, id.z, s.c0.z));
+  float3 cf = make_float3(fmaf(px, id.x, s.c1.x), fmaf(py, id.y, s.c1.y), fmaf(pz, id.z, s.c1.z));
+  const float3 e = make_float3(0x1p-20f * (fabsf(g.x) + fabsf(cn.x)), 0x1p-20f * (fabsf(g.y) + fabsf(cn.y)),
+                               0x1p-20f * (fabsf(g.z) + fabsf(cn.z)));
+  cn = cn - e;
+  cf = cf + e;
+  // near and far plane bytes per axis: (lo, hi) for a positive direction, swapped otherwise
+  const uint32_t nx0 = neg_x ? w3.z : w2.x, nx1 = neg_x ? w3.w : w2.y;
+  const uint32_t fx0 = neg_x ? w2.x : w3.z, fx1 = neg_x ? w2.y : w3.w;
+  const uint32_t ny0 = neg_y ? w4.x : w2.z, ny1 = neg_y ? w4.y : w2.w;
+  const uint32_t fy0 = neg_y ? w2.z : w4.x, fy1 = neg_y ? w2.w : w4.y;
+  const uint32_t nz0 = neg_z ? w4.z : w3.x, nz1 = neg_z ? w4.w : w3.y;
+  const uint32_t fz0 = neg_z ? w3.x : w4.z, fz1 = neg_z ? w3.y : w4.w;
+  uint32_t hit = 0u;   // slots whose boxes the query enters
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const uint32_t sel = 0x7604u | (uint32_t)(j & 3) << 4;   // (0, q, 0x80, 0x3F) of the word and 0x3F800000
+#define RR_WIDE_PLANE(w0_, w1_) __uint_as_float(__byte_perm(j < 4 ? w0_ : w1_, 0x3F800000u, sel))
+    const float lo = fmaxf(max3(fmaf(RR_WIDE_PLANE(nx0, nx1), g.x, cn.x), fmaf(RR_WIDE_PLANE(ny0, ny1), g.y, cn.y),
+                                fmaf(RR_WIDE_PLANE(nz0, nz1), g.z, cn.z)), s.t_min);
+    const float hi = fminf(min3(fmaf(RR_WIDE_PLANE(fx0, fx1), g.x, cf.x), fmaf(RR_WIDE_PLANE(fy0, fy1), g.y, cf.y),
+                                fmaf(RR_WIDE_PLANE(fz0, fz1), g.z, cf.z)), s.t_best);
+#undef RR_WIDE_PLANE
+    hit |= lo <= hi ? 1u << j : 0u;
+  }
+  hit &= w1.z;   // valid slots
+  const uint32_t imask = w0.w >> 24;
+  // internal hits in visiting order: bit k for slot k ^ octant
+  uint32_t in = hit & imask;
+  in = (oct & 1u) ? (in & 0x55u) << 1 | (in >> 1 & 0x55u) : in;
+  in = (oct & 2u) ? (in & 0x33u) << 2 | (in >> 2 & 0x33u) : in;
+  in = (oct & 4u) ? (in & 0x0Fu) << 4 | in >> 4 : in;
+  s.g_base = w1.x;
+  s.g_bits = imask << 8 | in;
+  s.t_base = w1.y;
+  s.t_bits = hit & ~imask;
+  s.t_counts = w1.w;
+}
+
+// the triangles of the next hit leaf slot
+template <bool kAny>
+__device__ __forceinline__ void step_wide_leaf(Trav& s, const ScanArgs& a, uint32_t& n_tris, bool count) {
+  const uint32_t j = __ffs(s.t_bits) - 1u;
+  s.t_bits &= s.t_bits - 1u;
+  const uint32_t below = s.t_counts & ((1u << (2u * j)) - 1u), n = s.t_counts >> (2u * j) & 3u;
+  const uint32_t first = s.t_base + __popc(below & 0x5555u) + 2u * __popc(below & 0xAAAAu);
+  for (uint32_t r = 0; r < n; ++r)
+    if (first + r < a.n_tris && trav_tri<kAny>(s, a, first + r, n_tris, count)) {
+      s.t_bits = 0u;
+      s.node = kNone;
+      break;
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -507,6 +528,7 @@ __device__ __noinline__ void settle_air_path(const ScanArgs& a, uint32_t bounce,
 // Binary nodes: 32 (batch of 24 scans of the 1M-triangle campus: 17.24 ms,
 // 17.65 at 16, 17.40 at 64); wide nodes: 16.
 constexpr int kSteps = 32, kStepsWide = 16;
+constexpr int kWideVisits = 2;   // wide nodes: visits per test of the waiting leaf slots
 // Binary nodes: node visits per triangle test.  A lane that reaches a leaf
 // waits until kNodeSteps visits of the others are over and the warp tests its
 // waiting leaves together: a query tests a triangle every 10 to 20 visits, so
@@ -514,11 +536,11 @@ constexpr int kSteps = 32, kStepsWide = 16;
 // three steps for one or two lanes (the same scans: 2 / 3 / 4 / 6 / 8 visits
 // 17.82 / 17.72 / 17.65 / 17.64 / 18.10 ms; one test per visit 22.53).
 constexpr int kNodeSteps = 4;
-// Binary stack: kNone, kStack entries, and room for the pushes of one group of
+// Traversal stack: the end mark, kStack entries, and room for the pushes of one group of
 // kNodeSteps visits, after which the query loop checks the depth.  The check
 // at every push and pop, with the divisions of trav_begin, was 6 % of a scan
 // (campus scan 1,134 -> 1,061 us, city scan 24.9 -> 23.4 ms).
-constexpr int kBinStack = 1 + kStack + kNodeSteps;
+constexpr int kQueryStack = 1 + kStack + kNodeSteps;
 // Resident threads per SM that the binary query kernels are compiled for:
 // 1,152 leaves 56 registers a thread.  Unbounded, the unrolled visits take 64
 // to 76 registers and lose more to occupancy than the spill-free code gains
@@ -553,7 +575,7 @@ __global__ void __launch_bounds__(kBlock, kWide ? 0 : kQueryThreads / kBlock) k_
   const uint32_t refill = a.refill;
   Trav s;
   s.node = kNone;
-  StackEntry stack[kWide ? kStack : kBinStack];
+  StackEntry stack[kQueryStack];
   uint32_t ray_i = kNone;   // ray of the lane's query (kNone: idle)
   float wa = 0.0f;          // any hit: W(omega_a) of the candidate
   uint32_t c_base = 0u, c_end = 0u;   // claimed, unassigned jobs (warp-uniform)
@@ -617,7 +639,8 @@ __global__ void __launch_bounds__(kBlock, kWide ? 0 : kQueryThreads / kBlock) k_
           // past t_lim no return can reach the image
           trav_begin(s, a, f3(ray.o_L), f3(ray.d_E), phys.x, (phys.w - ray.o_L.w) / n_cur, ray.meta.x, kWide);
         }
-        if (!kWide) bin_entry(reinterpret_cast<uint32_t*>(stack), 0) = kNone;
+        if (kWide) reinterpret_cast<uint2*>(stack)[0] = make_uint2(0u, 0u);
+        else bin_entry(reinterpret_cast<uint32_t*>(stack), 0) = kNone;
         if (!bvh_ok) s.node = kNone;
       }
     }
@@ -628,9 +651,19 @@ __global__ void __launch_bounds__(kBlock, kWide ? 0 : kQueryThreads / kBlock) k_
     }
     if (busy) {
       if (kWide) {
-#pragma unroll 2
-        for (int u = 0; u < kStepsWide && s.node != kNone; ++u)
-          step_wide<kAny>(s, reinterpret_cast<uint2*>(stack), a, n_nodes, n_tris, count);
+        uint2* st = reinterpret_cast<uint2*>(stack);
+#pragma unroll 1
+        for (int u = 0; u < kStepsWide && s.node != kNone; u += kWideVisits) {
+#pragma unroll
+          for (int v = 0; v < kWideVisits; ++v)
+            if (s.t_bits == 0u && s.node != kNone) step_wide_node<kAny>(s, st, a, n_nodes, count);
+          if (s.t_bits) step_wide_leaf<kAny>(s, a, n_tris, count);
+          if (s.sp > 1 + kStack) {   // deeper than the stack: the scan reports it
+            atomicOr(&a.ctr->error, kErrStack);
+            s.node = kNone;
+            s.t_bits = 0u;
+          }
+        }
       } else {
         uint32_t* st = reinterpret_cast<uint32_t*>(stack);
 #pragma unroll 1
