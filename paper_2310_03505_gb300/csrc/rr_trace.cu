@@ -28,7 +28,7 @@
 
 namespace rr {
 
-constexpr int kShadeBlock = 256;
+constexpr int kShadeTile = 256;   // rays of the smallest shading tile
 
 // ---------------------------------------------------------------------------
 // beam axis angle 2 pi a / n with an exact quadrant reduction; returns (cos, sin)
@@ -556,7 +556,7 @@ __global__ void __launch_bounds__(kBlock, kWide ? 0 : kQueryThreads / kBlock) k_
   uint32_t* ticket = kAny ? &C->vis_ticket[bounce] : &C->trace_ticket[bounce];
   const uint32_t gtid = blockIdx.x * blockDim.x + threadIdx.x, gsz = gridDim.x * blockDim.x;
   if (!kAny) {
-    const uint32_t tiles = (n + kShadeBlock - 1) / kShadeBlock;
+    const uint32_t tiles = (n + kShadeTile - 1) / kShadeTile;
     for (uint32_t t = gtid; t < tiles; t += gsz) a.tile_status[t] = 0ull;
     // the shading pass of this bounce counts the next bounce's rays per order bucket
     if (a.order_hist != nullptr && bounce + 1 <= RR_MAX_BOUNCES)
@@ -943,23 +943,30 @@ __device__ __forceinline__ float range_weight(const ScanDesc* sd, float r) {
   return (k != 0.0f && r > 1.0f) ? powf(r, -k) : 1.0f;
 }
 
-// The shading pass runs with 3 resident blocks per SM (80 registers) or 4
-// (64 registers, a few spilled).  Launch sequences with many rays take 4: the
-// more warps hide more of the random triangle and material loads (5M-triangle
-// city, 133k initial rays per sequence: 1.9 % per step).  Small ones take 3:
-// there the launch holds fewer tiles than the SMs have room for, each tile's
-// chain of dependent loads sets the time and the spills lengthen it (200k-
-// triangle campus, 27k initial rays per sequence: 1.4 %).
+// The shading pass runs in tiles of 256 rays with 3 resident blocks per SM (80
+// registers) or in tiles of 512 with 2 (64 registers, a few spilled).  Launch
+// sequences with many rays take the latter: more warps hide more of the random
+// triangle, material and lobe loads, and half as many tiles wait for their
+// predecessors (city scan 21.3 ms with tiles of 256, 21.0 with 512, 21.6 with
+// 128; 24 batched scans 14.4 / 14.2 / 14.7).  Small ones take the former:
+// there the launch holds fewer tiles than the SMs have room for and each tile's
+// chain of dependent loads sets the time (campus scan 1,008 us against 1,068).
+// What bounds it: 1,790 warp instructions per 32 rays at 19 of 32 lanes, the
+// barriers around the compaction first among the stalls (issue 40 %).  The
+// children and records stay in named registers until their places are known,
+// and the debug dump is compiled apart: indexed arrays of both kept 240 bytes
+// a thread in local memory (city scan 22.0 -> 21.3 ms, campus scan 1,039 ->
+// 1,017 us, 24 batched scans 15.0 -> 14.5 ms).
 constexpr uint32_t kShadeManyRays = 1u << 16;   // initial rays of a launch sequence
 
-template <int kMinBlocks>
-__global__ void __launch_bounds__(kShadeBlock, kMinBlocks) k_shade(ScanArgs a, uint32_t bounce) {
+template <int kBlock, int kMinBlocks, bool kDebug>
+__global__ void __launch_bounds__(kBlock, kMinBlocks) k_shade(ScanArgs a, uint32_t bounce) {
   __shared__ uint32_t s_tile;
-  __shared__ uint32_t s_wsum[kShadeBlock / 32];
+  __shared__ uint32_t s_wsum[kBlock / 32];
   __shared__ uint2 s_excl;
   extern __shared__ uint32_t s_hist[];   // [kOrderBuckets] children per order bucket (query order on only)
   const uint32_t n = a.ctr->count[bounce];
-  const uint32_t tiles = (n + kShadeBlock - 1) / kShadeBlock;
+  const uint32_t tiles = (n + kBlock - 1) / kBlock;
   const uint32_t rec0 = a.ctr->rec_start[bounce];
   const uint32_t seg0 = a.ctr->seg_start[bounce];
   const RayRec* qin = a.rays[bounce & 1];   // not restrict: deferred visibility writes its jobs over it
@@ -976,16 +983,20 @@ __global__ void __launch_bounds__(kShadeBlock, kMinBlocks) k_shade(ScanArgs a, u
   }
   const bool counting = a.order_key != nullptr && bounce + 1 < a.max_bounces;
   if (counting)
-    for (uint32_t j = threadIdx.x; j < kOrderBuckets; j += kShadeBlock) s_hist[j] = 0u;
+    for (uint32_t j = threadIdx.x; j < kOrderBuckets; j += kBlock) s_hist[j] = 0u;
   while (true) {
     if (threadIdx.x == 0) s_tile = atomicAdd(&a.ctr->shade_ticket[bounce], 1u);
     __syncthreads();
     const uint32_t tile = s_tile;
     if (tile >= tiles) break;
-    const uint32_t i = tile * kShadeBlock + threadIdx.x;
-    RayRec kid[2];
-    uint2 rec[2];
-    uint32_t nk = 0, nr = 0;
+    const uint32_t i = tile * kBlock + threadIdx.x;
+    // the children (reflected, refracted) and return records (traveled, air path), written once their places are known
+    bool sp_refl = false, sp_refr = false, rec_t = false, rec_a = false;
+    float3 p = make_float3(0.f, 0.f, 0.f), d_refl = p, d_refr = p;
+    float L1 = 0.f, e_refl = 0.f, e_refr = 0.f;
+    uint4 kmeta = make_uint4(0u, 0u, 0u, 0u);   // the reflected child's words; w of the refracted one: kmed
+    uint32_t kmed = 0u;
+    uint2 rt = make_uint2(0u, 0u), ra = rt;
     bool cand = false;           // an air-path candidate left to the visibility query (deferred visibility)
     int vj_kid = -1, vj_rec = -1;   // its child in kid[], its record in rec[] (-1: none)
     if (i < n) {
@@ -1014,9 +1025,9 @@ __global__ void __launch_bounds__(kShadeBlock, kMinBlocks) k_shade(ScanArgs a, u
         const float3 s_pos = f3(pr);
         const bool deeper = bounce + 1 < dims.z;
         const float t = h.t;
-        const float3 p = o + t * d;
+        p = o + t * d;
         const float n_cur = medium == kAir ? 1.0f : a.mats[medium].n;
-        const float L1 = ray.o_L.w + n_cur * t;
+        L1 = ray.o_L.w + n_cur * t;
         float E1 = E;
         if (medium != kAir) {
           const float alpha = kPi * n_cur * a.mats[medium].tan_d * phys.z / kC0;
@@ -1053,10 +1064,11 @@ __global__ void __launch_bounds__(kShadeBlock, kMinBlocks) k_shade(ScanArgs a, u
             can_refract = true;
           }
         }
-        const float3 d_refl = normalize(d + (2.0f * cos_i) * nrm);
+        d_refl = normalize(d + (2.0f * cos_i) * nrm);
         // traveled-path return: omega = theta0 + theta1 = 2 theta0, range L1
         const float theta0 = angle_between(d, -nrm);
-        const float ret_t = E1 * R * fminf(brdf_window(m, lut, 2.0f * theta0, beam.x), 1.0f);
+        const float E1R = E1 * R, E1T = E1 * T;
+        const float ret_t = E1R * fminf(brdf_window(m, lut, 2.0f * theta0, beam.x), 1.0f);
         float ret_a = 0.0f, range_a = 0.0f, e_rec = 0.0f;
         bool air_T = false;
         // the air-path candidate (Sec. III-A): its window W is open toward the
@@ -1089,12 +1101,12 @@ __global__ void __launch_bounds__(kShadeBlock, kMinBlocks) k_shade(ScanArgs a, u
         if (wag > 0.0f) {
           float base, cap;
           if (entering && medium == kAir) {
-            base = E1 * R;
-            cap = E1 * R - ret_t;
+            base = E1R;
+            cap = E1R - ret_t;
           } else {
             air_T = true;
-            base = E1 * T;
-            cap = E1 * T;
+            base = E1T;
+            cap = E1T;
           }
           ret_a = fmaxf(fminf(base * wag, cap), 0.0f);
           range_a = 0.5f * (L1 + length(s_pos - p));
@@ -1113,7 +1125,8 @@ __global__ void __launch_bounds__(kShadeBlock, kMinBlocks) k_shade(ScanArgs a, u
               float e = ret_t;
               if (rng.w & RR_SPECKLE) e *= -logf(u01(draw(rng, az, k, 1u | (((path << 8) | bounce) << 8)).x));
               e *= range_weight(sd, L1);
-              rec[nr++] = make_uint2(((offs.y + az - offs.w) << kBinBits) | (uint32_t)bin, __float_as_uint(e));
+              rec_t = true;
+              rt = make_uint2(((offs.y + az - offs.w) << kBinBits) | (uint32_t)bin, __float_as_uint(e));
             }
           }
           if (ret_a > 0.0f) {
@@ -1124,51 +1137,40 @@ __global__ void __launch_bounds__(kShadeBlock, kMinBlocks) k_shade(ScanArgs a, u
               e *= range_weight(sd, range_a);
               if (cand) {   // reserved with energy 0, written if the sensor is visible
                 e_rec = e;
-                vj_rec = (int)nr;
+                vj_rec = rec_t ? 1 : 0;
               }
-              rec[nr++] =
-                  make_uint2(((offs.y + az - offs.w) << kBinBits) | (uint32_t)bin, cand ? 0u : __float_as_uint(e));
+              rec_a = true;
+              ra = make_uint2(((offs.y + az - offs.w) << kBinBits) | (uint32_t)bin, cand ? 0u : __float_as_uint(e));
             }
           }
         }
-        const float e_refl = fmaxf(E1 * R - ret_t - (air_T ? 0.0f : ret_a_now), 0.0f);
-        const float e_refr = fmaxf(E1 * T - (air_T ? ret_a_now : 0.0f), 0.0f);
+        e_refl = fmaxf(E1R - ret_t - (air_T ? 0.0f : ret_a_now), 0.0f);
+        e_refr = fmaxf(E1T - (air_T ? ret_a_now : 0.0f), 0.0f);
         const bool in_range = L1 < pr.w;
-        const bool sp_refl = deeper && in_range && e_refl >= phys.y;
-        const bool sp_refr = deeper && in_range && can_refract && (rng.w & RR_REFRACTION) && e_refr >= phys.y;
+        sp_refl = deeper && in_range && e_refl >= phys.y;
+        sp_refr = deeper && in_range && can_refract && (rng.w & RR_REFRACTION) && e_refr >= phys.y;
         if (!sp_refl) tal[3] += e_refl;
         if (!sp_refr) tal[3] += e_refr;
-        const uint32_t mbit = ray.meta.z & 0x80000000u;
-        if (sp_refl) {
-          RayRec& c = kid[nk++];
-          c.o_L = make_float4(p.x, p.y, p.z, L1);
-          c.d_E = make_float4(d_refl.x, d_refl.y, d_refl.z, e_refl);
-          c.meta = make_uint4(h.leaf, ray.meta.y, mbit | (path << 1), (scan << 16) | medium);
-        }
-        if (sp_refr) {
-          const float3 d_refr = normalize(eta * d + (eta * cos_i - cos_t) * nrm);
-          RayRec& c = kid[nk++];
-          c.o_L = make_float4(p.x, p.y, p.z, L1);
-          c.d_E = make_float4(d_refr.x, d_refr.y, d_refr.z, e_refr);
-          c.meta = make_uint4(h.leaf, ray.meta.y, mbit | (path << 1) | 1u, (scan << 16) | next_med);
-        }
+        kmeta = make_uint4(h.leaf, ray.meta.y, (ray.meta.z & 0x80000000u) | (path << 1), (scan << 16) | medium);
+        kmed = (scan << 16) | next_med;
+        if (sp_refr) d_refr = normalize(eta * d + (eta * cos_i - cos_t) * nrm);
         if (cand) {   // the job, over this ray's record (read above, not read again)
           vj_kid = air_T ? (sp_refr ? (sp_refl ? 1 : 0) : -1) : (sp_refl ? 0 : -1);
           VisJob j;
           j.p_leaf = make_float4(p.x, p.y, p.z, __uint_as_float(h.leaf));
           j.idx = make_uint4(scan, kNone, kNone,
                              a.tallies != nullptr ? offs.x + (az - offs.w) * dims.y + k : kNone);
-          j.val = make_float4(air_T ? E1 * T : E1 * R - ret_t, ret_a, e_rec,
+          j.val = make_float4(air_T ? E1T : E1R - ret_t, ret_a, e_rec,
                               __uint_as_float(a.segs != nullptr ? seg0 + i : kNone));
           reinterpret_cast<VisJob*>(a.rays[bounce & 1])[i] = j;
         }
       }
-      if (a.tallies != nullptr) {
+      if (kDebug && a.tallies != nullptr) {
         float* tp = a.tallies + 4 * ((size_t)offs.x + (size_t)(az - offs.w) * dims.y + k);
         for (int q = 0; q < 4; ++q)
           if (tal[q] != 0.0f) atomicAdd(tp + q, tal[q]);
       }
-      if (a.segs != nullptr) {
+      if (kDebug && a.segs != nullptr) {
         const uint32_t si = seg0 + i;
         if (si < a.seg_cap) {
           rr_segment sg;
@@ -1191,6 +1193,7 @@ __global__ void __launch_bounds__(kShadeBlock, kMinBlocks) k_shade(ScanArgs a, u
       }
     }
     // block scan of (kids, recs)
+    const uint32_t nk = (sp_refl ? 1u : 0u) + (sp_refr ? 1u : 0u), nr = (rec_t ? 1u : 0u) + (rec_a ? 1u : 0u);
     const uint32_t packed = nk | (nr << 16);
     uint32_t x = packed;
     for (int off = 1; off < 32; off <<= 1) {
@@ -1200,7 +1203,7 @@ __global__ void __launch_bounds__(kShadeBlock, kMinBlocks) k_shade(ScanArgs a, u
     if (lane == 31) s_wsum[warp] = x;
     __syncthreads();
     uint32_t wpre = 0, total = 0;
-    for (int w2 = 0; w2 < kShadeBlock / 32; ++w2) {
+    for (int w2 = 0; w2 < kBlock / 32; ++w2) {
       const uint32_t v = s_wsum[w2];
       if (w2 < warp) wpre += v;
       total += v;
@@ -1233,24 +1236,29 @@ __global__ void __launch_bounds__(kShadeBlock, kMinBlocks) k_shade(ScanArgs a, u
         }
       }
     }
-    for (uint32_t c = 0; c < nk; ++c) {
-      const uint32_t pos = kbase + c;
-      if (pos < a.ray_cap) qout[pos] = kid[c];
-    }
-    if (a.order_key != nullptr && bounce + 1 < a.max_bounces) {
-      // order buckets of the children, counted in the block's histogram
-      for (uint32_t c = 0; c < nk; ++c) {
-        const uint32_t pos = kbase + c;
-        if (pos < a.ray_cap) {
+    RayRec kid[2];
+    kid[0].o_L = kid[1].o_L = make_float4(p.x, p.y, p.z, L1);
+    kid[0].d_E = make_float4(d_refl.x, d_refl.y, d_refl.z, e_refl);
+    kid[1].d_E = make_float4(d_refr.x, d_refr.y, d_refr.z, e_refr);
+    kid[0].meta = kmeta;
+    kid[1].meta = make_uint4(kmeta.x, kmeta.y, kmeta.z | 1u, kmed);
+    const bool counts = a.order_key != nullptr && bounce + 1 < a.max_bounces;
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      const uint32_t pos = kbase + (c && sp_refl ? 1u : 0u);
+      if ((c ? sp_refr : sp_refl) && pos < a.ray_cap) {
+        qout[pos] = kid[c];
+        if (counts) {   // order bucket of the child, counted in the block's histogram
           const uint32_t key = order_key(a, kid[c]);
           a.order_key[pos] = (uint16_t)key;
           atomicAdd(&s_hist[key], 1u);
         }
       }
     }
-    for (uint32_t c = 0; c < nr; ++c) {
-      const uint32_t pos = rec0 + rbase + c;
-      if (pos < a.rec_cap) a.recs[pos] = rec[c];
+    {
+      const uint32_t pos = rec0 + rbase;
+      if (rec_t && pos < a.rec_cap) a.recs[pos] = rt;
+      if (rec_a && pos + (rec_t ? 1u : 0u) < a.rec_cap) a.recs[pos + (rec_t ? 1u : 0u)] = ra;
     }
     if (tile == tiles - 1 && threadIdx.x == 0) {
       const uint32_t kids = ex.x + (total & 0xFFFFu), recs = ex.y + (total >> 16);
@@ -1278,7 +1286,7 @@ __global__ void __launch_bounds__(kShadeBlock, kMinBlocks) k_shade(ScanArgs a, u
   // with a barrier, so every count is in)
   if (counting) {
     uint32_t* h = a.order_hist + (size_t)(bounce + 1) * kOrderBuckets;
-    for (uint32_t j = threadIdx.x; j < kOrderBuckets; j += kShadeBlock)
+    for (uint32_t j = threadIdx.x; j < kOrderBuckets; j += kBlock)
       if (s_hist[j]) atomicAdd(&h[j], s_hist[j]);
   }
 }
@@ -1291,7 +1299,7 @@ using namespace rr;
 
 static int g_num_sms = 0;
 static int g_query_occ[2][2][3] = {{{0}}};   // [wide][any][block 64 / 128 / 256]
-static int g_shade_occ[2] = {0, 0};   // resident blocks of k_shade<3>, k_shade<4>
+static int g_shade_occ[2] = {0, 0};   // resident blocks of the small and large shading tiles
 
 static int block_index(uint32_t block) { return block <= 64u ? 0 : (block <= 128u ? 1 : 2); }
 
@@ -1318,8 +1326,9 @@ void init_dims() {
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   occ_all<false>(g_query_occ[0]);
   occ_all<true>(g_query_occ[1]);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&g_shade_occ[0], k_shade<3>, kShadeBlock, 0);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&g_shade_occ[1], k_shade<4>, kShadeBlock, 0);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&g_shade_occ[0], k_shade<kShadeTile, 3, false>, kShadeTile, 0);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&g_shade_occ[1], k_shade<2 * kShadeTile, 2, false>,
+                                                2 * kShadeTile, 0);
   for (int& o : g_shade_occ)
     if (o < 1) o = 1;
   g_num_sms = sms < 1 ? 1 : sms;
@@ -1388,10 +1397,12 @@ cudaError_t launch_order(const ScanArgs& a, uint32_t bounce, cudaStream_t st) {
 cudaError_t launch_shade(const ScanArgs& a, uint32_t bounce, cudaStream_t st) {
   init_dims();
   const size_t smem = a.order_key ? kOrderBuckets * sizeof(uint32_t) : 0;
-  if (a.n_rays0 >= kShadeManyRays)
-    k_shade<4><<<g_num_sms * g_shade_occ[1], kShadeBlock, smem, st>>>(a, bounce);
+  if (a.tallies != nullptr || a.segs != nullptr)
+    k_shade<kShadeTile, 3, true><<<g_num_sms * g_shade_occ[0], kShadeTile, smem, st>>>(a, bounce);
+  else if (a.n_rays0 >= kShadeManyRays)
+    k_shade<2 * kShadeTile, 2, false><<<g_num_sms * g_shade_occ[1], 2 * kShadeTile, smem, st>>>(a, bounce);
   else
-    k_shade<3><<<g_num_sms * g_shade_occ[0], kShadeBlock, smem, st>>>(a, bounce);
+    k_shade<kShadeTile, 3, false><<<g_num_sms * g_shade_occ[0], kShadeTile, smem, st>>>(a, bounce);
   return cudaGetLastError();
 }
 
