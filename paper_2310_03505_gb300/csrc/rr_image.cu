@@ -49,12 +49,18 @@ __device__ __forceinline__ int gauss_taps(float sigma, float* w) {
   return R;
 }
 
-// first record in [lo, hi) whose column is >= col (records are in column order)
+// first record in [lo, hi) whose column is >= col (records are in column
+// order), found by one warp: its lanes probe 32 places at once, so a list of a
+// million records takes 4 dependent loads where halving takes 20
 __device__ __forceinline__ uint32_t lower_col(const uint2* __restrict__ recs, uint32_t lo, uint32_t hi, uint32_t col) {
-  while (lo < hi) {
-    const uint32_t mid = lo + ((hi - lo) >> 1);
-    if ((__ldg(&recs[mid].x) >> kBinBits) < col) lo = mid + 1;
-    else hi = mid;
+  const uint32_t lane = threadIdx.x & 31u;
+  while (lo < hi) {   // the answer lies in [lo, hi]
+    const uint32_t step = (hi - lo + 31u) / 32u, at = lo + lane * step;
+    const bool below = at < hi && (__ldg(&recs[at].x) >> kBinBits) < col;
+    const uint32_t n = __popc(__ballot_sync(0xFFFFFFFFu, below));   // a prefix of the lanes
+    if (n == 0u) return lo;
+    hi = min(hi, lo + n * step);
+    lo += (n - 1u) * step + 1u;
   }
   return lo;
 }
@@ -133,35 +139,38 @@ __global__ void __launch_bounds__(kBlock) k_bin_column(ScanArgs a) {
   const float4 post = __ldg(&sd->post);   // blur sigma, pattern sigma, noise_sys, noise_amb
   const int lane = threadIdx.x & 31;
   for (uint32_t i = threadIdx.x; i < nb; i += blockDim.x) cells[i] = 0ull;
-  // record range of this column in every bounce's list: lane 2b / 2b+1
-  if (threadIdx.x < 32) {
-    const uint32_t b = (uint32_t)lane >> 1;
-    if (b < a.max_bounces) {
-      const uint32_t lo = a.ctr->rec_start[b], hi = a.ctr->rec_start[b + 1];
-      s_rng[lane] = lower_col(a.recs, lo, hi, c + (lane & 1));
-    }
+  // record range of this column in every bounce's list, one end a warp at a time
+  for (uint32_t q = threadIdx.x >> 5; q < 2u * a.max_bounces; q += kBlock / 32) {
+    const uint32_t r = lower_col(a.recs, a.ctr->rec_start[q >> 1], a.ctr->rec_start[(q >> 1) + 1], c + (q & 1u));
+    if (lane == 0) s_rng[q] = r;
   }
   __syncthreads();
-  for (uint32_t b = 0; b < a.max_bounces; ++b) {
-    const uint32_t lo = s_rng[2 * b], hi = s_rng[2 * b + 1];
-    // whole warps iterate together so that the shuffles see every lane
-    for (uint32_t base = lo; base < hi; base += blockDim.x) {
-      const uint32_t r = base + threadIdx.x;
-      bool valid = r < hi;
-      uint32_t bin = 0;
-      float e = 0.0f;
-      if (valid) {
-        const uint2 rc = __ldg(&a.recs[r]);
-        bin = rc.x & kBinMask;
-        e = __uint_as_float(rc.y);
-        valid = bin < nb;   // records always carry bin < n_bins; a failed scan may leave stale slots
-      }
-      const uint32_t tag = valid ? bin : 0x10000u + (uint32_t)lane;
-      const uint32_t peers = __match_any_sync(0xFFFFFFFFu, tag);
-      float2 acc = make_float2(0.0f, 0.0f);
-      for (uint32_t m = peers; m; m &= m - 1u) acc = neumaier(acc, __shfl_sync(peers, e, __ffs(m) - 1), 0.0f);
-      if (valid && lane == __ffs(peers) - 1) bin_add(&cells[bin], acc.x, acc.y);
+  // the column's records of all bounces in one run: a bounce's list alone
+  // seldom fills the block.  Whole warps iterate together so that the
+  // shuffles see every lane.
+  auto records = [&](uint32_t b) {   // a failed scan's stale slots need not be in order
+    return s_rng[2 * b + 1] > s_rng[2 * b] ? s_rng[2 * b + 1] - s_rng[2 * b] : 0u;
+  };
+  uint32_t total = 0;
+  for (uint32_t b = 0; b < a.max_bounces; ++b) total += records(b);
+  for (uint32_t base = 0; base < total; base += kBlock) {
+    uint32_t r = base + threadIdx.x;
+    bool valid = r < total;
+    uint32_t bin = 0;
+    float e = 0.0f;
+    if (valid) {
+      uint32_t b = 0;   // its bounce: r < total, so this ends at the last one
+      for (uint32_t n = records(0); r >= n; n = records(++b)) r -= n;
+      const uint2 rc = __ldg(&a.recs[s_rng[2 * b] + r]);
+      bin = rc.x & kBinMask;
+      e = __uint_as_float(rc.y);
+      valid = bin < nb;   // records always carry bin < n_bins; a failed scan may leave stale slots
     }
+    const uint32_t tag = valid ? bin : 0x10000u + (uint32_t)lane;
+    const uint32_t peers = __match_any_sync(0xFFFFFFFFu, tag);
+    float2 acc = make_float2(0.0f, 0.0f);
+    for (uint32_t m = peers; m; m &= m - 1u) acc = neumaier(acc, __shfl_sync(peers, e, __ffs(m) - 1), 0.0f);
+    if (valid && lane == __ffs(peers) - 1) bin_add(&cells[bin], acc.x, acc.y);
   }
   __syncthreads();
   for (uint32_t i = threadIdx.x; i < nb; i += blockDim.x) {
