@@ -21,6 +21,7 @@
 #include <cuda_runtime.h>
 
 #include <cstring>
+#include <mutex>
 
 #include "rr_host.h"
 
@@ -52,11 +53,12 @@ __device__ __forceinline__ int gauss_taps(float sigma, float* w) {
 // first record in [lo, hi) whose column is >= col (records are in column
 // order), found by one warp: its lanes probe 32 places at once, so a list of a
 // million records takes 4 dependent loads where halving takes 20
-__device__ __forceinline__ uint32_t lower_col(const uint2* __restrict__ recs, uint32_t lo, uint32_t hi, uint32_t col) {
+template <bool kRaw>
+__device__ __forceinline__ uint32_t lower_col(const ScanArgs& a, uint32_t lo, uint32_t hi, uint32_t col) {
   const uint32_t lane = threadIdx.x & 31u;
   while (lo < hi) {   // the answer lies in [lo, hi]
     const uint32_t step = (hi - lo + 31u) / 32u, at = lo + lane * step;
-    const bool below = at < hi && (__ldg(&recs[at].x) >> kBinBits) < col;
+    const bool below = at < hi && (kRaw ? __ldg(&a.raw_column[at]) : __ldg(&a.recs[at].x) >> kBinBits) < col;
     const uint32_t n = __popc(__ballot_sync(0xFFFFFFFFu, below));   // a prefix of the lanes
     if (n == 0u) return lo;
     hi = min(hi, lo + n * step);
@@ -123,7 +125,8 @@ __device__ __forceinline__ void bin_add(unsigned long long* cell, float x, float
 
 // A column is one block's work: with few columns the chip is filled by wider
 // blocks (launch_image).
-template <int kBlock>
+// kRaw: the returns are the caller's arrays (rr_accumulate_returns).
+template <int kBlock, bool kRaw>
 __global__ void __launch_bounds__(kBlock) k_bin_column(ScanArgs a) {
   extern __shared__ unsigned long long sm64[];
   unsigned long long* cells = sm64;                             // [n_bins] (sum, correction)
@@ -141,7 +144,7 @@ __global__ void __launch_bounds__(kBlock) k_bin_column(ScanArgs a) {
   for (uint32_t i = threadIdx.x; i < nb; i += blockDim.x) cells[i] = 0ull;
   // record range of this column in every bounce's list, one end a warp at a time
   for (uint32_t q = threadIdx.x >> 5; q < 2u * a.max_bounces; q += kBlock / 32) {
-    const uint32_t r = lower_col(a.recs, a.ctr->rec_start[q >> 1], a.ctr->rec_start[(q >> 1) + 1], c + (q & 1u));
+    const uint32_t r = lower_col<kRaw>(a, a.ctr->rec_start[q >> 1], a.ctr->rec_start[(q >> 1) + 1], c + (q & 1u));
     if (lane == 0) s_rng[q] = r;
   }
   __syncthreads();
@@ -161,10 +164,16 @@ __global__ void __launch_bounds__(kBlock) k_bin_column(ScanArgs a) {
     if (valid) {
       uint32_t b = 0;   // its bounce: r < total, so this ends at the last one
       for (uint32_t n = records(0); r >= n; n = records(++b)) r -= n;
-      const uint2 rc = __ldg(&a.recs[s_rng[2 * b] + r]);
-      bin = rc.x & kBinMask;
-      e = __uint_as_float(rc.y);
-      valid = bin < nb;   // records always carry bin < n_bins; a failed scan may leave stale slots
+      r += s_rng[2 * b];
+      if (kRaw) {
+        bin = __ldg(&a.raw_bin[r]);
+        e = __ldg(&a.raw_energy[r]);
+      } else {
+        const uint2 rc = __ldg(&a.recs[r]);
+        bin = rc.x & kBinMask;
+        e = __uint_as_float(rc.y);
+      }
+      valid = bin < nb;   // a caller's return past the image adds nothing; records always carry bin < n_bins; a failed scan may leave stale slots
     }
     const uint32_t tag = valid ? bin : 0x10000u + (uint32_t)lane;
     const uint32_t peers = __match_any_sync(0xFFFFFFFFu, tag);
@@ -230,18 +239,13 @@ __global__ void __launch_bounds__(kImgBlock) k_az_pattern(ScanArgs a) {
   sd->image[(size_t)az * nb + i] = acc;
 }
 
-// records of caller-given returns: (column << kBinBits | bin, energy); flags
-// a column that decreases or lies past the image
-__global__ void k_pack_returns(const uint32_t* __restrict__ column, const uint32_t* __restrict__ bin,
-                               const float* __restrict__ energy, uint32_t n, uint32_t n_columns, uint32_t n_bins,
-                               uint2* __restrict__ recs, uint32_t* __restrict__ bad) {
+// flags a column of caller-given returns that decreases or lies past the image
+__global__ void k_check_returns(const uint32_t* __restrict__ column, uint32_t n, uint32_t n_columns,
+                                uint32_t* __restrict__ bad) {
   const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= n) return;
-  const uint32_t c = column[k], b = bin[k];
+  const uint32_t c = column[k];
   if ((k > 0 && column[k - 1] > c) || c >= n_columns) atomicOr(bad, 1u);
-  // a bin past the image contributes nothing
-  const bool in = b < n_bins;
-  recs[k] = make_uint2(((c < n_columns ? c : 0u) << kBinBits) | (in ? b : 0u), in ? __float_as_uint(energy[k]) : 0u);
 }
 
 // Sec. III-B display mapping, one pixel: the reference form (a logarithm, a
@@ -310,7 +314,9 @@ static size_t bin_smem(uint32_t n_bins) { return (size_t)n_bins * (sizeof(unsign
 void init_image_attrs() {
   static bool attr_set = false;
   if (!attr_set) {
-    for (const void* k : {(const void*)k_bin_column<256>, (const void*)k_bin_column<512>, (const void*)k_bin_column<1024>})
+    for (const void* k : {(const void*)k_bin_column<256, false>, (const void*)k_bin_column<512, false>,
+                          (const void*)k_bin_column<1024, false>, (const void*)k_bin_column<256, true>,
+                          (const void*)k_bin_column<512, true>, (const void*)k_bin_column<1024, true>})
       cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bin_smem(RR_MAX_BINS));
     attr_set = true;
   }
@@ -319,9 +325,10 @@ void init_image_attrs() {
 cudaError_t launch_image(const ScanArgs& a, bool pattern, cudaStream_t st) {
   init_image_attrs();
   const uint32_t sms = (uint32_t)num_sms();
-  if (a.n_cols <= 2u * sms) k_bin_column<1024><<<a.n_cols, 1024, bin_smem(a.max_bins), st>>>(a);
-  else if (a.n_cols <= 4u * sms) k_bin_column<512><<<a.n_cols, 512, bin_smem(a.max_bins), st>>>(a);
-  else k_bin_column<256><<<a.n_cols, 256, bin_smem(a.max_bins), st>>>(a);
+  const int block = a.n_cols <= 2u * sms ? 1024 : (a.n_cols <= 4u * sms ? 512 : 256);
+  auto* bin = a.raw_column ? (block == 1024 ? k_bin_column<1024, true> : block == 512 ? k_bin_column<512, true> : k_bin_column<256, true>)
+                           : (block == 1024 ? k_bin_column<1024, false> : block == 512 ? k_bin_column<512, false> : k_bin_column<256, false>);
+  bin<<<a.n_cols, block, bin_smem(a.max_bins), st>>>(a);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   if (pattern) {
@@ -373,6 +380,53 @@ static bool usable_here(const void* p) {
   return at.type == cudaMemoryTypeDevice && at.device == dev;
 }
 
+// Setup block of a call whose buffers are all used in place: slots compiled
+// into the library (an allocation of a few hundred bytes took most of the call,
+// the driver maps and unmaps its 2 MiB block around it).  A slot is held for
+// one blocking call; with none free the call allocates.
+namespace {
+struct Setup {
+  ScanCounters ctr;
+  ScanDesc desc;
+  uint32_t pre[4], bad;   // ray prefix (unused) and column prefix; the check's flag
+};
+constexpr int kSetupSlots = 16, kSetupDevices = 64;
+__device__ __align__(256) unsigned char g_setup[kSetupSlots][(sizeof(Setup) + 255) & ~size_t(255)];
+std::mutex g_setup_lock;
+uint32_t g_setup_used[kSetupDevices];
+char* g_setup_base[kSetupDevices];
+
+class SetupSlot {
+ public:
+  SetupSlot() {
+    std::lock_guard<std::mutex> guard(g_setup_lock);
+    if (cudaGetDevice(&dev_) != cudaSuccess || dev_ < 0 || dev_ >= kSetupDevices) {
+      cudaGetLastError();
+      return;
+    }
+    void* p = g_setup_base[dev_];
+    if (!p && cudaGetSymbolAddress(&p, g_setup) != cudaSuccess) {
+      cudaGetLastError();
+      return;
+    }
+    g_setup_base[dev_] = static_cast<char*>(p);
+    for (int k = 0; k < kSetupSlots && slot_ < 0; ++k)
+      if (!(g_setup_used[dev_] >> k & 1u)) slot_ = k;
+    if (slot_ >= 0) g_setup_used[dev_] |= 1u << slot_;
+  }
+  ~SetupSlot() {
+    std::lock_guard<std::mutex> guard(g_setup_lock);
+    if (slot_ >= 0) g_setup_used[dev_] &= ~(1u << slot_);
+  }
+  SetupSlot(const SetupSlot&) = delete;
+  SetupSlot& operator=(const SetupSlot&) = delete;
+  void* get() const { return slot_ >= 0 ? g_setup_base[dev_] + slot_ * sizeof g_setup[0] : nullptr; }
+
+ private:
+  int dev_ = -1, slot_ = -1;
+};
+}  // namespace
+
 extern "C" int rr_accumulate_returns(const uint32_t* column, const uint32_t* bin, const float* energy, uint64_t n,
                                      uint32_t n_columns, uint32_t n_bins, float* out) {
   if (!out || (n && (!column || !bin || !energy))) return fail(RR_ERR_INVALID_ARG, "NULL buffer");
@@ -383,44 +437,42 @@ extern "C" int rr_accumulate_returns(const uint32_t* column, const uint32_t* bin
   const size_t img_bytes = (size_t)n_columns * n_bins * sizeof(float);
   // Buffers of this device are read and written where they are; others (host
   // memory, another device's, or not aligned to their elements) go through
-  // the scratch of this call, one allocation: [column][bin][energy][records]
-  // [image][setup].  Nine allocations and the copies of device inputs were
-  // most of a call.
-  const bool own_col = usable_here(column), own_bin = usable_here(bin), own_e = usable_here(energy),
-             own_out = usable_here(out);
-  const size_t nn = n ? n : 1;
-  struct Setup {
-    ScanCounters ctr;
-    ScanDesc desc;
-    uint32_t pre[4], bad;   // ray prefix (unused) and column prefix; the check's flag
+  // the scratch of this call, one allocation (none when all are): [column][bin][energy][image]
+  // [setup].  Nine allocations, the copies of device inputs and their packing
+  // into records were most of a call (1.5M returns into 400 columns: 679 us).
+  const bool own_col = usable_here(column), own_bin = usable_here(bin), own_e = usable_here(energy);
+  // an image over its own inputs is made apart
+  auto over_out = [&](const void* p) {
+    const uintptr_t i0 = reinterpret_cast<uintptr_t>(p), o0 = reinterpret_cast<uintptr_t>(out);
+    return i0 < o0 + img_bytes && o0 < i0 + n * 4;
   };
+  const bool own_out = usable_here(out) && !over_out(column) && !over_out(bin) && !over_out(energy);
+  const size_t nn = n ? n : 1;
   auto up = [](size_t x) { return (x + 255) & ~size_t(255); };
   const size_t in_bytes = up(nn * 4);
   size_t off = 0, o_col = 0, o_bin = 0, o_e = 0, o_img = 0;
   if (!own_col) o_col = off, off += in_bytes;
   if (!own_bin) o_bin = off, off += in_bytes;
   if (!own_e) o_e = off, off += in_bytes;
-  const size_t o_recs = off;
-  off += up(nn * 8);
   if (!own_out) o_img = off, off += up(img_bytes);
+  const SetupSlot slot;   // given back after the last wait of every path below
   const size_t o_setup = off;
-  off += up(sizeof(Setup));
+  if (!slot.get()) off += up(sizeof(Setup));
   char* w = nullptr;
-  cudaError_t e = dev_malloc(&w, off);
+  cudaError_t e = off ? dev_malloc(&w, off) : cudaSuccess;
   if (e != cudaSuccess) {
     cudaGetLastError();
     return cuda_fail(e, "accumulating the returns");
   }
   auto cleanup = [&]() {
     cudaStreamSynchronize(st);
-    cudaFree(w);
+    if (w) cudaFree(w);
   };
   const uint32_t* d_col = own_col ? column : (const uint32_t*)(w + o_col);
   const uint32_t* d_bin = own_bin ? bin : (const uint32_t*)(w + o_bin);
   const float* d_e = own_e ? energy : (const float*)(w + o_e);
-  uint2* d_recs = (uint2*)(w + o_recs);
   float* d_img = own_out ? out : (float*)(w + o_img);
-  Setup* d_setup = (Setup*)(w + o_setup);
+  Setup* d_setup = (Setup*)(slot.get() ? slot.get() : w + o_setup);
   if (n && !own_col) e = cudaMemcpyAsync(w + o_col, column, n * 4, cudaMemcpyDefault, st);
   if (e == cudaSuccess && n && !own_bin) e = cudaMemcpyAsync(w + o_bin, bin, n * 4, cudaMemcpyDefault, st);
   if (e == cudaSuccess && n && !own_e) e = cudaMemcpyAsync(w + o_e, energy, n * 4, cudaMemcpyDefault, st);
@@ -433,8 +485,7 @@ extern "C" int rr_accumulate_returns(const uint32_t* column, const uint32_t* bin
   setup.ctr.rec_start[1] = (uint32_t)n;
   if (e == cudaSuccess) e = cudaMemcpyAsync(d_setup, &setup, sizeof setup, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess && n) {
-    k_pack_returns<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(d_col, d_bin, d_e, (uint32_t)n, n_columns, n_bins,
-                                                                 d_recs, &d_setup->bad);
+    k_check_returns<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(d_col, (uint32_t)n, n_columns, &d_setup->bad);
     e = cudaGetLastError();
   }
   // the check's answer before anything is written to the output
@@ -459,9 +510,10 @@ extern "C" int rr_accumulate_returns(const uint32_t* column, const uint32_t* bin
   a.n_cols = n_columns;
   a.max_bounces = 1;
   a.max_bins = n_bins;
-  a.recs = d_recs;
+  a.raw_column = d_col;
+  a.raw_bin = d_bin;
+  a.raw_energy = d_e;
   a.ctr = &d_setup->ctr;
-  a.rec_cap = (uint32_t)nn;
   e = launch_image(a, false, st);
   if (e == cudaSuccess && !own_out) e = cudaMemcpyAsync(out, d_img, img_bytes, cudaMemcpyDefault, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
@@ -470,6 +522,6 @@ extern "C" int rr_accumulate_returns(const uint32_t* column, const uint32_t* bin
     cleanup();
     return cuda_fail(e, "accumulating the returns");
   }
-  cudaFree(w);
+  if (w) cudaFree(w);
   return RR_OK;
 }

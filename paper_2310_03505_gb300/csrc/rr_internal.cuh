@@ -187,6 +187,10 @@ struct ScanArgs {
   RayRec* rays[2];
   HitRec* hits;
   uint2* recs;               // (column << kBinBits | bin, energy bits)
+  // the same as the caller's own arrays (rr_accumulate_returns; then recs is not used)
+  const uint32_t* raw_column;
+  const uint32_t* raw_bin;
+  const float* raw_energy;
   unsigned long long* tile_status;
   ScanCounters* ctr;
   float* image_tmp;          // images before the azimuth pattern (or null)

@@ -63,6 +63,12 @@ def test_binning_routes(rrlib, n_columns, where):
     rr.rr_accumulate_returns(*arrs, n_columns, n_bins, out)
     got = out.cpu().numpy() if on[3] else out
     assert np.all(np.abs(got.astype(np.float64) - ref) <= ULPS * ulp32(ref))
+    if where == "device" and n_columns * n_bins <= e.size * 4:   # an image over its own inputs
+        room = torch.zeros(max(e.size, n_columns * n_bins), device="cuda")
+        room[:e.size] = arrs[2]
+        rr.rr_accumulate_returns(arrs[0], arrs[1], room[:e.size], n_columns, n_bins,
+                                 room[:n_columns * n_bins].view(n_columns, n_bins))
+        assert torch.equal(room[:n_columns * n_bins].view(n_columns, n_bins).cpu(), torch.from_numpy(got))
     # a refused call leaves a device output as it was
     bad = torch.from_numpy(col.copy()).cuda()
     bad[-1] = n_columns
