@@ -125,9 +125,9 @@ constexpr int kWideNodeWords = 5;
 // the L1 and L2 footprint), and one byte permutation per plane picks the near
 // or far plane and decodes it, where the float form needed a min and a max.
 constexpr int kNodeWords = 2;
-// The grid of a scene's binary nodes, two float4: (base x, y, z, 0), (scale x, y, z, 0)
+// The grid of a scene's binary nodes, three float4: (base x, y, z, 0), (scale x, y, z, 0), (1 / scale, 0)
 constexpr int kFrameWord = 16;        // its place in the build status words (rr_scene::d_misc)
-constexpr int kMiscWords = 24;        // 0..5 centroid bounds, 6 error bits, 7 depth, 8..13 vertex bounds, 16..23 the frame
+constexpr int kMiscWords = 28;        // 0..5 centroid bounds, 6 error bits, 7 depth, 8..13 vertex bounds, 16..27 the frame
 
 // Return record key: global image column (scan's first column + azimuth)
 // and range bin.  Records of one bounce are in column order.
