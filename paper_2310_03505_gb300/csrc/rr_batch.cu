@@ -377,6 +377,14 @@ static int graph_launch(rr_scene* s, ExecCtx* x, const ScanArgs& a, bool pattern
   return RR_OK;
 }
 
+// Lanes of a query warp that take rays.  A launch sequence of a few thousand
+// rays leaves most of the chip without a warp while its own warps run through
+// the union of 32 rays' visits: fewer rays a warp shorten that, until the
+// warps no longer fit beside each other (tiny room scan of 3,200 rays 191 us
+// with 32 lanes, 183 with 16, 177 with 8; campus scan of 12,000 rays 610 / 611
+// / 652).
+static uint32_t query_lanes(uint32_t rays) { return rays <= 4096u ? 8u : (rays <= 8192u ? 16u : 32u); }
+
 int batch_enqueue(rr_scene* s, ExecCtx* x, const rr_pose* poses, const rr_sensor_params* ps, float* const* images,
                   uint32_t n, const DebugOut* dbg, cudaStream_t st, void* ws, const WsLayout& L, bool profile,
                   bool allow_graph, const LaunchCfg& cfg, void* host_desc, const uint32_t* az_range) {
@@ -473,7 +481,8 @@ int batch_enqueue(rr_scene* s, ExecCtx* x, const rr_pose* poses, const rr_sensor
   // return: with a min_energy cut the return decides, so the query runs first
   a.defer_vis = (any_flags & RR_MULTIPATH) && maxb > 1 && !min_energy ? 1u : 0u;
   a.vis_list = (uint32_t*)(w + L.off_vis);
-  a.refill = cfg.refill;
+  a.lanes = cfg.trace_block == 64u && !(any_flags & RR_COUNT_TRAVERSAL) ? query_lanes(rays) : 32u;
+  a.refill = std::min(cfg.refill, a.lanes);
   a.rays[0] = (rr::RayRec*)(w + L.off_rays0);
   a.rays[1] = (rr::RayRec*)(w + L.off_rays1);
   a.hits = (rr::HitRec*)(w + L.off_hits);

@@ -183,6 +183,7 @@ struct ScanArgs {
   uint32_t max_bins;         // over the batch
   uint32_t any_flags;        // union of the scans' flags
   uint32_t refill;           // a warp hands out new queries once this many lanes are idle (1..32)
+  uint32_t lanes;            // lanes of a warp that take queries (fewer in small launch sequences)
   // workspace
   RayRec* rays[2];
   HitRec* hits;

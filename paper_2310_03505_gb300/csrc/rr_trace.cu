@@ -21,6 +21,7 @@
 // sequence of launches with no host round trip between bounces.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstring>
 #include <type_traits>
 
@@ -470,7 +471,6 @@ __device__ __forceinline__ void step_wide_leaf(Trav& s, const ScanArgs& a, uint3
 // ahead of the shading pass.  Persistent: a warp claims jobs in chunks and hands
 // them to its idle lanes once at least `refill` lanes are idle (or all are),
 // so the lanes stay busy however uneven the query lengths are.
-constexpr uint32_t kClaim = 32;
 
 // Receive-beam weight of a return from p (Sec. III-A air path): g =
 // exp(-delta^2 / 2 sigma^2), delta the angle between p - sensor and the beam
@@ -548,7 +548,9 @@ constexpr int kQueryStack = 1 + kStack + kNodeSteps;
 constexpr int kQueryThreads = 1152;
 // kCount: the traversal counters (RR_COUNT_TRAVERSAL) are compiled only into
 // the kernels of the scans that ask for them
-template <bool kAny, int kBlock, bool kWide, bool kCount>
+// kSpread: only a.lanes lanes of a warp take queries (small launch sequences);
+// apart, because the whole-warp kernels lose 1 % to the extra operands.
+template <bool kAny, int kBlock, bool kWide, bool kCount, bool kSpread>
 __global__ void __launch_bounds__(kBlock, kWide ? 0 : kQueryThreads / kBlock) k_query(ScanArgs a, uint32_t bounce) {
   typedef typename std::conditional<kWide, uint2, uint32_t>::type StackEntry;
   ScanCounters* C = a.ctr;
@@ -572,7 +574,10 @@ __global__ void __launch_bounds__(kBlock, kWide ? 0 : kQueryThreads / kBlock) k_
   constexpr bool count = kCount;
   const int lane = threadIdx.x & 31;
   const uint32_t lt = (1u << lane) - 1u;
-  const uint32_t refill = a.refill;
+  const uint32_t refill = a.refill;   // at most a.lanes
+  // the other lanes leave, the votes and shuffles below go on among the rest
+  // (lane 0 always stays)
+  if (kSpread && (uint32_t)lane >= a.lanes) return;
   Trav s;
   s.node = kNone;
   StackEntry stack[kQueryStack];
@@ -593,7 +598,7 @@ __global__ void __launch_bounds__(kBlock, kWide ? 0 : kQueryThreads / kBlock) k_
         c_base += need;
       } else {
         c_base = c_end;
-        const uint32_t more = need - avail, chunk = max(more, kClaim);
+        const uint32_t more = need - avail, chunk = max(more, kSpread ? a.lanes : 32u);
         uint32_t b = 0;
         if (lane == 0) b = atomicAdd(ticket, chunk);
         b = __shfl_sync(0xFFFFFFFFu, b, 0);
@@ -712,16 +717,20 @@ __global__ void __launch_bounds__(kBlock, kWide ? 0 : kQueryThreads / kBlock) k_
       }
     }
   }
-  // counters, one atomic per warp
-  for (int off = 16; off > 0; off >>= 1) n_done += __shfl_xor_sync(0xFFFFFFFFu, n_done, off);
-  if (lane == 0 && n_done) atomicAdd(kAny ? &C->stat_anyhit : &C->stat_closest, (unsigned long long)n_done);
+  // counters, one atomic per warp (per lane where the warp is not whole)
+  constexpr bool whole = !kSpread;
+  if (whole)
+    for (int off = 16; off > 0; off >>= 1) n_done += __shfl_xor_sync(0xFFFFFFFFu, n_done, off);
+  if ((lane == 0 || !whole) && n_done)
+    atomicAdd(kAny ? &C->stat_anyhit : &C->stat_closest, (unsigned long long)n_done);
   if (count) {
     unsigned long long nn = n_nodes, nt = n_tris;
-    for (int off = 16; off > 0; off >>= 1) {
-      nn += __shfl_xor_sync(0xFFFFFFFFu, nn, off);
-      nt += __shfl_xor_sync(0xFFFFFFFFu, nt, off);
-    }
-    if (lane == 0) {
+    if (whole)
+      for (int off = 16; off > 0; off >>= 1) {
+        nn += __shfl_xor_sync(0xFFFFFFFFu, nn, off);
+        nt += __shfl_xor_sync(0xFFFFFFFFu, nt, off);
+      }
+    if (lane == 0 || !whole) {
       atomicAdd(kAny ? &C->stat_nodes_any : &C->stat_nodes, nn);
       atomicAdd(kAny ? &C->stat_tris_any : &C->stat_tris, nt);
     }
@@ -1305,7 +1314,7 @@ static int block_index(uint32_t block) { return block <= 64u ? 0 : (block <= 128
 
 template <bool kAny, int kBlock, bool kWide>
 static void occ_of(int* out) {
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, k_query<kAny, kBlock, kWide, false>, kBlock, 0);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, k_query<kAny, kBlock, kWide, false, false>, kBlock, 0);
   if (*out < 1) *out = 1;
 }
 
@@ -1352,9 +1361,14 @@ cudaError_t launch_raygen(const ScanArgs& a, cudaStream_t st) {
 
 template <bool kAny, bool kWide, bool kCount>
 static void query_launch_c(const ScanArgs& a, uint32_t bounce, int bi, int grid, cudaStream_t st) {
-  if (bi == 0) k_query<kAny, 64, kWide, kCount><<<grid, 64, 0, st>>>(a, bounce);
-  else if (bi == 1) k_query<kAny, 128, kWide, kCount><<<grid, 128, 0, st>>>(a, bounce);
-  else k_query<kAny, 256, kWide, kCount><<<grid, 256, 0, st>>>(a, bounce);
+  if (bi == 0) {
+    if (a.lanes < 32u && !kCount) k_query<kAny, 64, kWide, false, true><<<grid, 64, 0, st>>>(a, bounce);
+    else k_query<kAny, 64, kWide, kCount, false><<<grid, 64, 0, st>>>(a, bounce);
+  } else if (bi == 1) {
+    k_query<kAny, 128, kWide, kCount, false><<<grid, 128, 0, st>>>(a, bounce);
+  } else {
+    k_query<kAny, 256, kWide, kCount, false><<<grid, 256, 0, st>>>(a, bounce);
+  }
 }
 template <bool kAny, bool kWide>
 static void query_launch(const ScanArgs& a, uint32_t bounce, int bi, int grid, cudaStream_t st) {
@@ -1370,7 +1384,9 @@ cudaError_t launch_query(const ScanArgs& a, uint32_t bounce, bool any, const Lau
   const int bi = block_index(c.trace_block);
   int per_sm = g_query_occ[wide ? 1 : 0][any ? 1 : 0][bi];
   if (c.trace_blocks_per_sm > 0 && (int)c.trace_blocks_per_sm < per_sm) per_sm = (int)c.trace_blocks_per_sm;
-  const int grid = g_num_sms * per_sm;
+  // no more blocks than the bounce can have queries (each ray has two children at most)
+  const uint64_t warps = (((uint64_t)a.n_rays0 << bounce) + a.lanes - 1) / a.lanes, per_block = 2u << bi;
+  const int grid = (int)std::max<uint64_t>(1, std::min<uint64_t>((uint64_t)g_num_sms * per_sm, (warps + per_block - 1) / per_block));
   if (wide) {
     if (any) query_launch<true, true>(a, bounce, bi, grid, st);
     else query_launch<false, true>(a, bounce, bi, grid, st);
@@ -1397,12 +1413,15 @@ cudaError_t launch_order(const ScanArgs& a, uint32_t bounce, cudaStream_t st) {
 cudaError_t launch_shade(const ScanArgs& a, uint32_t bounce, cudaStream_t st) {
   init_dims();
   const size_t smem = a.order_key ? kOrderBuckets * sizeof(uint32_t) : 0;
+  const uint64_t most = (uint64_t)a.n_rays0 << bounce;   // rays of the bounce
+  const int small = (int)std::max<uint64_t>(
+      1, std::min<uint64_t>((uint64_t)g_num_sms * g_shade_occ[0], (most + kShadeTile - 1) / kShadeTile));
   if (a.tallies != nullptr || a.segs != nullptr)
-    k_shade<kShadeTile, 3, true><<<g_num_sms * g_shade_occ[0], kShadeTile, smem, st>>>(a, bounce);
+    k_shade<kShadeTile, 3, true><<<small, kShadeTile, smem, st>>>(a, bounce);
   else if (a.n_rays0 >= kShadeManyRays)
     k_shade<2 * kShadeTile, 2, false><<<g_num_sms * g_shade_occ[1], 2 * kShadeTile, smem, st>>>(a, bounce);
   else
-    k_shade<kShadeTile, 3, false><<<g_num_sms * g_shade_occ[0], kShadeTile, smem, st>>>(a, bounce);
+    k_shade<kShadeTile, 3, false><<<small, kShadeTile, smem, st>>>(a, bounce);
   return cudaGetLastError();
 }
 
