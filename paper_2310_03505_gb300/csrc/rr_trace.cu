@@ -184,6 +184,20 @@ __device__ __forceinline__ float min3(float a, float b, float c) {
   return d;
 }
 
+// two fmas in one instruction: (a, b) * (m, m) + c, c a packed pair
+__device__ __forceinline__ unsigned long long pack2(float a, float b) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ float2 fma2(float a, float b, float m, unsigned long long c) {
+  unsigned long long r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(pack2(a, b)), "l"(pack2(m, m)), "l"(c));
+  float2 o;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(o.x), "=f"(o.y) : "l"(r));
+  return o;
+}
+
 // ---------------------------------------------------------------------------
 // Resumable traversal.  A query (closest hit, or any hit for visibility) is
 // advanced one step at a time -- one node visit or one triangle test -- so
@@ -409,12 +423,12 @@ __device__ __forceinline__ void step_wide_node(Trav& s, uint2* stack, const Scan
   const float px = fmaf(sx, 8355840.0f, __uint_as_float(w0.x)), py = fmaf(sy, 8355840.0f, __uint_as_float(w0.y)),
               pz = fmaf(sz, 8355840.0f, __uint_as_float(w0.z));
   const float3 g = make_float3(32768.0f * sx * id.x, 32768.0f * sy * id.y, 32768.0f * sz * id.z);
-  float3 cn = make_float3(fmaf(px, id.x, s.c0.x), fmaf(py, id.y, s.c0.y), fmaf(pz, id.z, s.c0.z));
-  float3 cf = make_float3(fmaf(px, id.x, s.c1.x), fmaf(py, id.y, s.c1.y), fmaf(pz, id.z, s.c1.z));
+  const float3 cn = make_float3(fmaf(px, id.x, s.c0.x), fmaf(py, id.y, s.c0.y), fmaf(pz, id.z, s.c0.z));
+  const float3 cf = make_float3(fmaf(px, id.x, s.c1.x), fmaf(py, id.y, s.c1.y), fmaf(pz, id.z, s.c1.z));
   const float3 e = make_float3(0x1p-20f * (fabsf(g.x) + fabsf(cn.x)), 0x1p-20f * (fabsf(g.y) + fabsf(cn.y)),
                                0x1p-20f * (fabsf(g.z) + fabsf(cn.z)));
-  cn = cn - e;
-  cf = cf + e;
+  const unsigned long long cx = pack2(cn.x - e.x, cf.x + e.x), cy = pack2(cn.y - e.y, cf.y + e.y),
+                           cz = pack2(cn.z - e.z, cf.z + e.z);
   // near and far plane bytes per axis: (lo, hi) for a positive direction, swapped otherwise
   const uint32_t nx0 = neg_x ? w3.z : w2.x, nx1 = neg_x ? w3.w : w2.y;
   const uint32_t fx0 = neg_x ? w2.x : w3.z, fx1 = neg_x ? w2.y : w3.w;
@@ -427,10 +441,12 @@ __device__ __forceinline__ void step_wide_node(Trav& s, uint2* stack, const Scan
   for (int j = 0; j < 8; ++j) {
     const uint32_t sel = 0x7604u | (uint32_t)(j & 3) << 4;   // (0, q, 0x80, 0x3F) of the word and 0x3F800000
 #define RR_WIDE_PLANE(w0_, w1_) __uint_as_float(__byte_perm(j < 4 ? w0_ : w1_, 0x3F800000u, sel))
-    const float lo = fmaxf(max3(fmaf(RR_WIDE_PLANE(nx0, nx1), g.x, cn.x), fmaf(RR_WIDE_PLANE(ny0, ny1), g.y, cn.y),
-                                fmaf(RR_WIDE_PLANE(nz0, nz1), g.z, cn.z)), s.t_min);
-    const float hi = fminf(min3(fmaf(RR_WIDE_PLANE(fx0, fx1), g.x, cf.x), fmaf(RR_WIDE_PLANE(fy0, fy1), g.y, cf.y),
-                                fmaf(RR_WIDE_PLANE(fz0, fz1), g.z, cf.z)), s.t_best);
+    // (near, far) of an axis in one packed fma: 3 % of a scan over these nodes
+    // (the binary step, with two boxes a visit, gets 2 % slower by it)
+    const float2 vx = fma2(RR_WIDE_PLANE(nx0, nx1), RR_WIDE_PLANE(fx0, fx1), g.x, cx);
+    const float2 vy = fma2(RR_WIDE_PLANE(ny0, ny1), RR_WIDE_PLANE(fy0, fy1), g.y, cy);
+    const float2 vz = fma2(RR_WIDE_PLANE(nz0, nz1), RR_WIDE_PLANE(fz0, fz1), g.z, cz);
+    const float lo = fmaxf(max3(vx.x, vy.x, vz.x), s.t_min), hi = fminf(min3(vx.y, vy.y, vz.y), s.t_best);
 #undef RR_WIDE_PLANE
     hit |= lo <= hi ? 1u << j : 0u;
   }
