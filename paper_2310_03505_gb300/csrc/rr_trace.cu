@@ -142,7 +142,9 @@ __device__ __forceinline__ WoopRay make_woop(float3 o, float3 d) {
 // watertight test; returns t (or -1) -- products are kept unfused so that a
 // shared edge evaluates to exactly opposite values in both triangles
 // (the vertices in the ray's frame: the triangle copy w.rot)
-__device__ __forceinline__ float woop_hit(const WoopRay& w, float3 v0, float3 v1, float3 v2) {
+// (edge: the hit lies within 2^-10 of the triangle's edges)
+__device__ __forceinline__ float woop_hit(const WoopRay& w, float3 v0, float3 v1, float3 v2, bool& edge) {
+  edge = false;
   const float3 A = v0 - w.o, B = v1 - w.o, C = v2 - w.o;
   const float Az_ = A.z, Bz_ = B.z, Cz_ = C.z;
   const float Ax = __fsub_rn(A.x, __fmul_rn(w.Sx, Az_));
@@ -158,7 +160,37 @@ __device__ __forceinline__ float woop_hit(const WoopRay& w, float3 v0, float3 v1
   const float det = U + V + W;
   if (det == 0.0f) return -1.0f;
   const float T = U * (w.Sz * Az_) + V * (w.Sz * Bz_) + W * (w.Sz * Cz_);
+  edge = fminf(fminf(fabsf(U), fabsf(V)), fabsf(W)) <= 0x1p-10f * fabsf(det);
   return T / det;
+}
+
+// Where two triangles share an edge, the test above takes the ray that meets it
+// for both, at distances that differ in their last bits, and takes rays a
+// rounding error beside an outer edge.  Which of these count is decided by the
+// triangle's own float box, not by the coarser boxes of the nodes: a hit next
+// to an edge stands only if the robust slab test of that box (planes at
+// fma(b, 1/d, -o/d) moved apart by 4 u |o/d|, far planes inflated by 1 + 2
+// gamma_3) accepts the ray up to the best hit so far.  So the same one of two
+// such triangles is found whatever the nodes' grid (one path in some 10^8
+// queries turned at a building's edge without it; 4 % of a scan).  Apart from
+// the loop, for its registers: inlined it costs 2 % more.  v, o and d in the
+// frame of the triangle copy.
+constexpr float kBoxInflate = 1.00000036f;   // 1 + 2 gamma_3 (Ize 2013)
+__device__ __noinline__ bool edge_hit_stands(float3 v0, float3 v1, float3 v2, float3 o, float3 d, float t_min,
+                                             float t_best) {
+  float lo = -INFINITY, hi = INFINITY;
+  const float b0[3] = {fminf(fminf(v0.x, v1.x), v2.x), fminf(fminf(v0.y, v1.y), v2.y), fminf(fminf(v0.z, v1.z), v2.z)};
+  const float b1[3] = {fmaxf(fmaxf(v0.x, v1.x), v2.x), fmaxf(fmaxf(v0.y, v1.y), v2.y), fmaxf(fmaxf(v0.z, v1.z), v2.z)};
+  const float oo[3] = {o.x, o.y, o.z}, dd[3] = {d.x, d.y, d.z};
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const float id = __fdiv_rn(1.0f, fabsf(dd[k]) > 1e-30f ? dd[k] : copysignf(1e-30f, dd[k]));
+    const float od = __fmul_rn(oo[k], id), e = copysignf(0x1p-22f * fabsf(od), id);
+    const float t0 = fmaf(b0[k], id, __fsub_rn(-od, e)), t1 = fmaf(b1[k], id, __fadd_rn(-od, e));
+    lo = fmaxf(lo, fminf(t0, t1));
+    hi = fminf(hi, fmaxf(t0, t1));
+  }
+  return fmaxf(lo, t_min) <= fminf(__fmul_rn(hi, kBoxInflate), t_best);
 }
 
 // Selectors of a binary node's box word: __byte_perm(word, 0x3F000000, sel)
@@ -285,15 +317,37 @@ __device__ __forceinline__ void trav_begin(Trav& s, const ScanArgs& a, float3 o,
   }
 }
 
-// triangle j against the query; returns true when an any-hit query is answered
+// Binary nodes: node visits per triangle test.  A lane that reaches a leaf
+// waits until kNodeSteps visits of the others are over and the warp tests its
+// waiting leaves together: a query tests a triangle every 10 to 20 visits, so
+// testing each at once sent the whole warp through the triangle test in two of
+// three steps for one or two lanes (the same scans: 2 / 3 / 4 / 6 / 8 visits
+// 17.82 / 17.72 / 17.65 / 17.64 / 18.10 ms; one test per visit 22.53).
+constexpr int kNodeSteps = 4;
+// Traversal stack: the end mark, kStack entries, and room for the pushes of one group of
+// kNodeSteps visits, after which the query loop checks the depth.  The check
+// at every push and pop, with the divisions of trav_begin, was 6 % of a scan
+// (campus scan 1,134 -> 1,061 us, city scan 24.9 -> 23.4 ms).
+// Binary: the ray's direction follows (for edge_hit_stands, out of the registers).
+constexpr int kQueryStack = 1 + kStack + kNodeSteps;
+
+// triangle j against the query; returns true when an any-hit query is
+// answered.  dir: the ray's direction (binary nodes), null: any edge hit stands
+// (the wide nodes' boxes).
 template <bool kAny>
-__device__ __forceinline__ bool trav_tri(Trav& s, const ScanArgs& a, uint32_t j, uint32_t& n_tris, bool count) {
+__device__ __forceinline__ bool trav_tri(Trav& s, const ScanArgs& a, uint32_t j, uint32_t& n_tris, bool count,
+                                         const uint32_t* dir) {
   if (j == s.skip) return false;
   if (count) ++n_tris;
   const float4* tp = a.tri + a.tri_copy * s.w.rot + 3 * (size_t)j;
   const float4 v0 = __ldg(tp), v1 = __ldg(tp + 1), v2 = __ldg(tp + 2);
-  const float t = woop_hit(s.w, f3(v0), f3(v1), f3(v2));
+  bool edge;
+  const float t = woop_hit(s.w, f3(v0), f3(v1), f3(v2), edge);
   if (t > s.t_min) {
+    if (dir != nullptr && edge && t <= s.t_best) {
+      const float3 d = make_float3(__uint_as_float(dir[0]), __uint_as_float(dir[1]), __uint_as_float(dir[2]));
+      if (!edge_hit_stands(f3(v0), f3(v1), f3(v2), s.w.o, tri_rotate(d, s.w.rot), s.t_min, s.t_best)) return false;
+    }
     if (kAny) {
       if (t < s.t_best) {
         s.best = j;
@@ -358,7 +412,7 @@ __device__ __forceinline__ void step_inner(Trav& s, uint32_t* stack, const ScanA
 // Binary BVH: one leaf
 template <bool kAny>
 __device__ __forceinline__ void step_leaf(Trav& s, uint32_t* stack, const ScanArgs& a, uint32_t& n_tris, bool count) {
-  if (trav_tri<kAny>(s, a, s.node & ~kLeafBit, n_tris, count)) {
+  if (trav_tri<kAny>(s, a, s.node & ~kLeafBit, n_tris, count, stack + kQueryStack)) {
     s.node = kNone;
   } else {
     s.sp -= 4;
@@ -472,7 +526,7 @@ __device__ __forceinline__ void step_wide_leaf(Trav& s, const ScanArgs& a, uint3
   const uint32_t below = s.t_counts & ((1u << (2u * j)) - 1u), n = s.t_counts >> (2u * j) & 3u;
   const uint32_t first = s.t_base + __popc(below & 0x5555u) + 2u * __popc(below & 0xAAAAu);
   for (uint32_t r = 0; r < n; ++r)
-    if (first + r < a.n_tris && trav_tri<kAny>(s, a, first + r, n_tris, count)) {
+    if (first + r < a.n_tris && trav_tri<kAny>(s, a, first + r, n_tris, count, nullptr)) {
       s.t_bits = 0u;
       s.node = kNone;
       break;
@@ -545,18 +599,6 @@ __device__ __noinline__ void settle_air_path(const ScanArgs& a, uint32_t bounce,
 // 17.65 at 16, 17.40 at 64); wide nodes: 16.
 constexpr int kSteps = 32, kStepsWide = 16;
 constexpr int kWideVisits = 2;   // wide nodes: visits per test of the waiting leaf slots
-// Binary nodes: node visits per triangle test.  A lane that reaches a leaf
-// waits until kNodeSteps visits of the others are over and the warp tests its
-// waiting leaves together: a query tests a triangle every 10 to 20 visits, so
-// testing each at once sent the whole warp through the triangle test in two of
-// three steps for one or two lanes (the same scans: 2 / 3 / 4 / 6 / 8 visits
-// 17.82 / 17.72 / 17.65 / 17.64 / 18.10 ms; one test per visit 22.53).
-constexpr int kNodeSteps = 4;
-// Traversal stack: the end mark, kStack entries, and room for the pushes of one group of
-// kNodeSteps visits, after which the query loop checks the depth.  The check
-// at every push and pop, with the divisions of trav_begin, was 6 % of a scan
-// (campus scan 1,134 -> 1,061 us, city scan 24.9 -> 23.4 ms).
-constexpr int kQueryStack = 1 + kStack + kNodeSteps;
 // Resident threads per SM that the binary query kernels are compiled for:
 // 1,152 leaves 56 registers a thread.  Unbounded, the unrolled visits take 64
 // to 76 registers and lose more to occupancy than the spill-free code gains
@@ -596,7 +638,7 @@ __global__ void __launch_bounds__(kBlock, kWide ? 0 : kQueryThreads / kBlock) k_
   if (kSpread && (uint32_t)lane >= a.lanes) return;
   Trav s;
   s.node = kNone;
-  StackEntry stack[kQueryStack];
+  StackEntry stack[kWide ? kQueryStack : kQueryStack + 3];
   uint32_t ray_i = kNone;   // ray of the lane's query (kNone: idle)
   float wa = 0.0f;          // any hit: W(omega_a) of the candidate
   uint32_t c_base = 0u, c_end = 0u;   // claimed, unassigned jobs (warp-uniform)
@@ -628,6 +670,7 @@ __global__ void __launch_bounds__(kBlock, kWide ? 0 : kQueryThreads / kBlock) k_
         }
       }
       if (job != kNone) {
+        float3 dir;
         if (kAny && a.defer_vis) {
           ray_i = a.vis_list[job];
           const float4 pl = reinterpret_cast<const VisJob*>(q)[ray_i].p_leaf;
@@ -636,7 +679,8 @@ __global__ void __launch_bounds__(kBlock, kWide ? 0 : kQueryThreads / kBlock) k_
           const float3 p = f3(pl);
           const float3 v = f3(__ldg(&sd->pos_rmax)) - p;
           const float dist = length(v);
-          trav_begin(s, a, p, (1.0f / dist) * v, __ldg(&sd->phys.x), dist, __float_as_uint(pl.w), kWide);
+          dir = (1.0f / dist) * v;
+          trav_begin(s, a, p, dir, __ldg(&sd->phys.x), dist, __float_as_uint(pl.w), kWide);
         } else if (kAny) {
           const uint2 jb = jobs[job];
           ray_i = jb.x;
@@ -649,7 +693,8 @@ __global__ void __launch_bounds__(kBlock, kWide ? 0 : kQueryThreads / kBlock) k_
           const float3 p = o + h.t * d;
           const float3 v = f3(__ldg(&sd->pos_rmax)) - p;
           const float dist = length(v);
-          trav_begin(s, a, p, (1.0f / dist) * v, __ldg(&sd->phys.x), dist, h.leaf, kWide);
+          dir = (1.0f / dist) * v;
+          trav_begin(s, a, p, dir, __ldg(&sd->phys.x), dist, h.leaf, kWide);
         } else {
           ray_i = perm ? perm[job] : job;
           if (ray_i >= n) ray_i = job;   // only after a failed shading pass (the scan reports it)
@@ -658,10 +703,18 @@ __global__ void __launch_bounds__(kBlock, kWide ? 0 : kQueryThreads / kBlock) k_
           const float4 phys = __ldg(&a.desc[sm.x].phys);   // t_min, min_energy, freq, r_lim
           const float n_cur = sm.y == kAir ? 1.0f : __ldg(&a.mats[sm.y].n);
           // past t_lim no return can reach the image
-          trav_begin(s, a, f3(ray.o_L), f3(ray.d_E), phys.x, (phys.w - ray.o_L.w) / n_cur, ray.meta.x, kWide);
+          dir = f3(ray.d_E);
+          trav_begin(s, a, f3(ray.o_L), dir, phys.x, (phys.w - ray.o_L.w) / n_cur, ray.meta.x, kWide);
         }
-        if (kWide) reinterpret_cast<uint2*>(stack)[0] = make_uint2(0u, 0u);
-        else bin_entry(reinterpret_cast<uint32_t*>(stack), 0) = kNone;
+        if (kWide) {
+          reinterpret_cast<uint2*>(stack)[0] = make_uint2(0u, 0u);
+        } else {
+          uint32_t* st = reinterpret_cast<uint32_t*>(stack);
+          st[0] = kNone;
+          st[kQueryStack] = __float_as_uint(dir.x);
+          st[kQueryStack + 1] = __float_as_uint(dir.y);
+          st[kQueryStack + 2] = __float_as_uint(dir.z);
+        }
         if (!bvh_ok) s.node = kNone;
       }
     }
