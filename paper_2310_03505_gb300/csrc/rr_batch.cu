@@ -546,10 +546,13 @@ int batch_run(rr_scene* s, ExecCtx* x, const rr_pose* poses, const rr_sensor_par
 // queries), the extra launches and the joins cost more.  Measured, split in 3
 // against whole: tiny room 3,200 rays 217 / 183 us and 40,000 rays 320 / 277;
 // 200k-triangle campus 12,000 rays 596 / 550, 24,000 rays 669 / 693, 40,000
-// rays 789 / 868; 5M-triangle city 24,000 rays 1,119 / 1,251.
+// rays 789 / 868; 5M-triangle city 24,000 rays 1,119 / 1,251.  The limit
+// counts per range, so a scan whose whole ray tree does not fit it stays split:
+// its ranges may hold what the whole would have to drop.
 static bool scan_whole(const rr_scene* s, const rr_sensor_params* p) {
   const uint64_t rays = (uint64_t)p->n_azimuth * p->rays_per_beam;
-  return rays < (1u << 14) || (s->nt < (1u << 13) && rays < (1u << 16));
+  if (rays >= (1u << 14) && (s->nt >= (1u << 13) || rays >= (1u << 16))) return false;
+  return !plan_workspace(p, 1, s->cfg.ws_limit, nullptr, s->cfg.order == RR_ORDER_CELL_OCTANT).clamped;
 }
 
 // One scan as split_streams azimuth ranges, each a launch sequence of its own

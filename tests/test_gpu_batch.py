@@ -248,6 +248,26 @@ def test_split_scan_equals_whole(tiny_scene, variant):
         rr.rr_batch_config_set(h, **saved)
 
 
+def test_default_split_stays_within_the_workspace_limit(tiny_scene):
+    """A small scan runs whole by default only if its whole ray tree fits the
+    workspace limit: under a limit that holds each of the three ranges but not
+    the whole, the default still succeeds (run whole, the scan is refused)."""
+    _, pz, base, h = tiny_scene
+    p = scenes.sensor(**{**base, "n_azimuth": 400, "rays_per_beam": 64})
+    ref = alone(h, pz, p)
+    _, limit = rr.rr_batch_plan([{**p, "n_azimuth": 134}])
+    saved = rr.rr_batch_config_get(h)
+    try:
+        rr.rr_batch_config_set(h, workspace_limit=limit, split_streams=1)
+        with pytest.raises(rr.RRError) as e:
+            alone(h, pz, p)
+        assert e.value.code == rr.RR_ERR_CAPACITY
+        rr.rr_batch_config_set(h, workspace_limit=limit, split_streams=0)
+        assert_close(alone(h, pz, p), ref, "default split under the limit")
+    finally:
+        rr.rr_batch_config_set(h, **saved)
+
+
 def test_profile_busy_time(tiny_scene):
     """rr_profile_read's busy_ms is the union of a kind's launch intervals: on
     one stream the launches of a kind never overlap, so it equals the summed
