@@ -394,7 +394,6 @@ constexpr int kSetupSlots = 16, kSetupDevices = 64;
 __device__ __align__(256) unsigned char g_setup[kSetupSlots][(sizeof(Setup) + 255) & ~size_t(255)];
 std::mutex g_setup_lock;
 uint32_t g_setup_used[kSetupDevices];
-char* g_setup_base[kSetupDevices];
 
 class SetupSlot {
  public:
@@ -404,12 +403,13 @@ class SetupSlot {
       cudaGetLastError();
       return;
     }
-    void* p = g_setup_base[dev_];
-    if (!p && cudaGetSymbolAddress(&p, g_setup) != cudaSuccess) {
+    // asked for on each call: a device reset moves the symbol
+    void* p = nullptr;
+    if (cudaGetSymbolAddress(&p, g_setup) != cudaSuccess) {
       cudaGetLastError();
       return;
     }
-    g_setup_base[dev_] = static_cast<char*>(p);
+    base_ = static_cast<char*>(p);
     for (int k = 0; k < kSetupSlots && slot_ < 0; ++k)
       if (!(g_setup_used[dev_] >> k & 1u)) slot_ = k;
     if (slot_ >= 0) g_setup_used[dev_] |= 1u << slot_;
@@ -420,9 +420,10 @@ class SetupSlot {
   }
   SetupSlot(const SetupSlot&) = delete;
   SetupSlot& operator=(const SetupSlot&) = delete;
-  void* get() const { return slot_ >= 0 ? g_setup_base[dev_] + slot_ * sizeof g_setup[0] : nullptr; }
+  void* get() const { return slot_ >= 0 ? base_ + slot_ * sizeof g_setup[0] : nullptr; }
 
  private:
+  char* base_ = nullptr;
   int dev_ = -1, slot_ = -1;
 };
 }  // namespace
