@@ -47,6 +47,7 @@ METRIC = "Mrays/s (all bounces) & scans/s on 1 GB300; p50/p99 served scan latenc
 RAY_IO_BYTES = 48 + 16          # ray record read + hit record written per closest-hit query
 NODE_BYTES, TRI_BYTES = 32, 48  # BVH node and triangle record
 L2_FLUSH_NOTE = "flushed between steps (256 MiB write, outside the timed events)"
+SPLIT_DEFAULT = 3               # azimuth ranges of a scan of this size by the library's default
 ORDER_DEFAULT = "queue"         # the library's default query order (rr_batch_config.query_order)
 
 
@@ -499,7 +500,8 @@ def plain_bench(rr, device, stream, flush, sc, pz, params, steps, warmup, *, ran
                                    else rr.RR_ORDER_QUEUE)
         cfg = rr.rr_batch_config_get(h)
         nf = "wide8_q8" if cfg["node_format"] == rr.RR_NODES_WIDE8 else "binary_fp32"
-        out.update(node_format=nf, split_streams=cfg["split_streams"], workspace_limit=cfg["workspace_limit"],
+        out.update(node_format=nf, split_streams=cfg["split_streams"] or SPLIT_DEFAULT,
+                   workspace_limit=cfg["workspace_limit"],
                    query_order="cell_octant" if cfg["query_order"] == rr.RR_ORDER_CELL_OCTANT else "queue")
         img = torch.zeros(params["n_azimuth"], params["n_bins"], device=device)
         warm_ids, step_ids = shard_scan_ids(rank, steps, warmup)
@@ -695,7 +697,6 @@ def main():
     from paper_2310_03505_gb300 import scenes
     sc, pz, params = scenes.config_medium() if args.no_large else scenes.config_large()
     workload = MEDIUM_WORKLOAD if args.no_large else LARGE_WORKLOAD
-    split_default = 3
 
     if args.impl == "reference":
         # the oracle arm: rank 0 only, on the host cores
@@ -709,7 +710,7 @@ def main():
                 "steps": args.steps, "warmup": args.warmup, "ms_per_step": 1e3 * t_step,
                 "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "f64",
                 "data": "synthetic",
-                "config": headline_config(sc, params, nf, split_default, args.step_bvh, args.gpus,
+                "config": headline_config(sc, params, nf, SPLIT_DEFAULT, args.step_bvh, args.gpus,
                                           ORDER_DEFAULT if args.query_order == "auto" else args.query_order,
                                           workload),
                 "cpu_baseline": {"value": value, "unit": "Mrays/s", "cores": cores, "kind": "oracle",

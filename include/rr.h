@@ -391,12 +391,12 @@ int rr_scan_batch_async(rr_scene* scene, uint32_t n, const rr_pose* poses, const
    split_streams        rr_scan / rr_scan_async trace a scan as this many
                         azimuth ranges, each on its own stream, so that the
                         slow queries closing one range's bounce overlap the
-                        other ranges' work (1..4; 0: the default, 3).  Scans
-                        with a beam pattern run whole, and while the value is
-                        the default so do scans too small to gain from it
-                        (unless the whole ray tree exceeds workspace_limit,
-                        which counts per range).  The image is the same up to
-                        the rounding of the bin sums.
+                        other ranges' work (1..4: exactly that many; 0, the
+                        default, as rr_batch_config_get reports it: 3, and 1
+                        for scans too small to gain from a split, unless the
+                        whole ray tree exceeds workspace_limit, which counts
+                        per range).  Scans with a beam pattern run whole.  The
+                        image is the same up to the rounding of the bin sums.
    bvh_build            RR_BVH_SAH_TOP (default): the LBVH (Morton codes,
                         radix sort, Karras hierarchy, refit) with the part
                         above its subtrees of at most 32 triangles rebuilt

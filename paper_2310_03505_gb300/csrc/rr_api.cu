@@ -592,7 +592,8 @@ int rr_scene_set_lobe(rr_scene* s, uint32_t material, const float* density) {
 // The checksum is FNV-1a (64 bit) over the payload.
 struct SceneBlobHeader {
   char magic[8];            // "RRSCENE" and a zero byte
-  uint32_t version, nv, nt, nm, n_tab, reserved;
+  uint32_t version, nv, nt, nm, n_tab;
+  uint32_t config_rev;      // 1: split_streams 0 stands for the default; 0: written as 3, as was every default
   uint64_t payload_bytes, checksum;
   uint8_t pad[16];
 };
@@ -652,6 +653,7 @@ int rr_scene_save(const rr_scene* s, void* blob, uint64_t capacity, uint64_t* si
   h.nt = s->nt;
   h.nm = s->nm;
   h.n_tab = n_tab;
+  h.config_rev = 1;
   h.payload_bytes = payload;
   h.checksum = fnv1a(b, payload);
   memcpy(blob, &h, sizeof h);
@@ -691,6 +693,7 @@ int rr_scene_load(const void* blob, uint64_t size, rr_scene** out) {
   rr_batch_config cfg;
   memcpy(&cfg, q, sizeof cfg);
   q += sizeof cfg;
+  if (h.config_rev == 0 && cfg.split_streams == kDefaultSplit) cfg.split_streams = 0;
   rr_scene* s = nullptr;
   int rc = rr_scene_create(vtx.data(), h.nv, tri.data(), h.nt, mid.data(), mats.data(), h.nm, &s);
   if (rc != RR_OK) return rc;

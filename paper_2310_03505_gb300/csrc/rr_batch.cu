@@ -562,8 +562,8 @@ static bool scan_whole(const rr_scene* s, const rr_sensor_params* p) {
 // Scans with a beam pattern (which needs every column) run whole.
 int scan_split(rr_scene* s, const rr_pose* pose, const rr_sensor_params* p, float* image, cudaStream_t st,
                bool profile) {
-  uint32_t k_n = std::min<uint32_t>(s->cfg.split, p->n_azimuth);
-  if (s->cfg.split_auto && scan_whole(s, p)) k_n = 1;
+  const uint32_t asked = s->cfg.split ? s->cfg.split : (scan_whole(s, p) ? 1u : kDefaultSplit);
+  const uint32_t k_n = std::min<uint32_t>(asked, p->n_azimuth);
   if (k_n <= 1 || p->az_pattern_sigma > 0.f) {
     float* const images[1] = {image};
     return batch_run(s, &s->main, pose, p, images, 1, nullptr, st, s->cfg);
@@ -661,7 +661,7 @@ static LaunchCfg cfg_from_abi(const rr_batch_config* c) {
   o.node_format = c->node_format;
   o.refill = c->refill_threshold ? c->refill_threshold : 16u;
   if (c->workspace_limit) o.ws_limit = c->workspace_limit;
-  o.split = c->split_streams ? c->split_streams : 3u;
+  o.split = c->split_streams;
   o.bvh_build = c->bvh_build;
   o.order = c->query_order;
   return o;
@@ -740,10 +740,7 @@ int rr_batch_config_set(rr_scene* s, const rr_batch_config* c) {
   const int rc = cfg_check(c);
   if (rc != RR_OK) return rc;
   const bool rebuild = c->bvh_build != s->cfg.bvh_build;
-  // a split_streams that was not changed from the default stays a default
-  const bool split_auto = c->split_streams == 0 || (s->cfg.split_auto && c->split_streams == s->cfg.split);
   s->cfg = cfg_from_abi(c);
-  s->cfg.split_auto = split_auto;
   return rebuild ? rebuild_bvh(s, current_stream()) : RR_OK;
 }
 

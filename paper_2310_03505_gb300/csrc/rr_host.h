@@ -30,14 +30,14 @@ struct LaunchCfg {
   uint32_t use_graph = 1;             // capture each launch sequence once and replay it
   uint32_t node_format = RR_NODES_BINARY;
   uint32_t refill = 16;               // idle lanes that trigger a refill (1..32)
-  uint32_t split = 3;                 // a single scan as this many azimuth ranges on their own streams
-  bool split_auto = true;             // split is the library's default: small scans run whole (scan_whole)
+  uint32_t split = 0;                 // a single scan as this many azimuth ranges on their own streams;
+                                      // 0: kDefaultSplit, small scans whole (scan_whole)
   uint64_t ws_limit = uint64_t(24) << 30;
   uint32_t bvh_build = RR_BVH_SAH_TOP;
   uint32_t order = 0;                 // RR_ORDER_*: query order of the closest-hit queries of bounces >= 1
 };
 
-constexpr uint32_t kMaxSplit = 4;
+constexpr uint32_t kMaxSplit = 4, kDefaultSplit = 3;
 
 // What one stream of scans needs besides the scene: device counters and
 // status, the scan workspace, an image buffer for host outputs, pinned

@@ -296,3 +296,44 @@ def test_profile_busy_time(tiny_scene):
             assert rr.rr_profile_read(h)["trace"] == (0.0, 0, 0.0)   # the reset cleared it
     finally:
         rr.rr_batch_config_set(h, **saved)
+
+
+def test_split_streams_default_and_explicit(tiny_scene):
+    """split_streams 0 is the library's choice (a small scan runs whole) and is
+    what rr_batch_config_get reports for it; any other value is followed, 3 on
+    a fresh scene too.  Getting the configuration, setting another number and
+    setting the first back restores the choice, and so does a blob, one written
+    when the default was stored as 3 included."""
+    sc, pz, base, _ = tiny_scene
+    p = scenes.sensor(**base)
+
+    def ranges(h):
+        alone(h, pz, p)
+        rr.rr_profile_read(h, reset=True)
+        rr.rr_profile_enable(h, True)
+        alone(h, pz, p)
+        rr.rr_profile_enable(h, False)
+        launches = rr.rr_profile_read(h, reset=True)["trace"][1]
+        assert launches % p["max_bounces"] == 0
+        return launches // p["max_bounces"]
+
+    fresh = P.gpu_scene(sc)
+    loaded = []
+    try:
+        saved = rr.rr_batch_config_get(fresh)
+        assert saved["split_streams"] == 0 and ranges(fresh) == 1
+        blob = rr.rr_scene_save(fresh)
+        rr.rr_batch_config_set(fresh, split_streams=3)
+        assert rr.rr_batch_config_get(fresh)["split_streams"] == 3 and ranges(fresh) == 3
+        explicit = rr.rr_scene_save(fresh)
+        rr.rr_batch_config_set(fresh, split_streams=1)
+        rr.rr_batch_config_set(fresh, **saved)
+        assert rr.rr_batch_config_get(fresh) == saved and ranges(fresh) == 1
+        # the header's word at 28 tells how the blob stores a default
+        old = explicit[:28] + bytes(4) + explicit[32:]
+        for b, split, n in ((blob, 0, 1), (explicit, 3, 3), (old, 0, 1)):
+            loaded.append(rr.rr_scene_load(b))
+            assert rr.rr_batch_config_get(loaded[-1])["split_streams"] == split and ranges(loaded[-1]) == n
+    finally:
+        for h in [fresh] + loaded:
+            rr.rr_scene_destroy(h)
