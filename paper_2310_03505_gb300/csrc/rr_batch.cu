@@ -377,13 +377,20 @@ static int graph_launch(rr_scene* s, ExecCtx* x, const ScanArgs& a, bool pattern
   return RR_OK;
 }
 
-// Lanes of a query warp that take rays.  A launch sequence of a few thousand
-// rays leaves most of the chip without a warp while its own warps run through
-// the union of 32 rays' visits: fewer rays a warp shorten that, until the
-// warps no longer fit beside each other (tiny room scan of 3,200 rays 191 us
-// with 32 lanes, 183 with 16, 177 with 8; campus scan of 12,000 rays 610 / 611
-// / 652).
-static uint32_t query_lanes(uint32_t rays) { return rays <= 4096u ? 8u : (rays <= 8192u ? 16u : 32u); }
+// Lanes of a query warp that take rays.  A scan of a few thousand rays leaves
+// most of the chip without a warp while its own warps run through the union of
+// 32 rays' visits: fewer rays a warp shorten that, until the warps no longer
+// fit beside each other.  rays: those in flight together, all ranges of a
+// split scan.  Whole scans over 5 bounces, 8 / 16 / 32 lanes, in us:
+//   rays    room             200k campus      5M city
+//   400     236 / 244 / 251  348 / 361 / 376  362 / 376 / 392
+//   3,200   259 / 266 / 269  408 / 413 / 423  435 / 446 / 457
+//   4,000   258 / 261 / 269  424 / 428 / 436  445 / 452 / 456
+//   6,000   271 / 274 / 270  453 / 452 / 444  478 / 481 / 482
+//   8,000   295 / 288 / 273  492 / 487 / 461  507 / 507 / 486
+// and in three ranges of 4,000 (12,000 rays) 320 / 307 / 302, 528 / 483 / 469,
+// 540 / 522 / 515: 16 lanes are never the best.
+static uint32_t query_lanes(uint64_t rays) { return rays <= 5120u ? 8u : 32u; }
 
 int batch_enqueue(rr_scene* s, ExecCtx* x, const rr_pose* poses, const rr_sensor_params* ps, float* const* images,
                   uint32_t n, const DebugOut* dbg, cudaStream_t st, void* ws, const WsLayout& L, bool profile,
@@ -481,7 +488,8 @@ int batch_enqueue(rr_scene* s, ExecCtx* x, const rr_pose* poses, const rr_sensor
   // return: with a min_energy cut the return decides, so the query runs first
   a.defer_vis = (any_flags & RR_MULTIPATH) && maxb > 1 && !min_energy ? 1u : 0u;
   a.vis_list = (uint32_t*)(w + L.off_vis);
-  a.lanes = cfg.trace_block == 64u && !(any_flags & RR_COUNT_TRAVERSAL) ? query_lanes(rays) : 32u;
+  const uint64_t in_flight = az_range ? (uint64_t)ps[0].n_azimuth * ps[0].rays_per_beam : rays;
+  a.lanes = cfg.trace_block == 64u && !(any_flags & RR_COUNT_TRAVERSAL) ? query_lanes(in_flight) : 32u;
   a.refill = std::min(cfg.refill, a.lanes);
   a.rays[0] = (rr::RayRec*)(w + L.off_rays0);
   a.rays[1] = (rr::RayRec*)(w + L.off_rays1);

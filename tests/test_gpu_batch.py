@@ -337,3 +337,28 @@ def test_split_streams_default_and_explicit(tiny_scene):
     finally:
         for h in [fresh] + loaded:
             rr.rr_scene_destroy(h)
+
+
+@pytest.mark.parametrize("n_az,rays", [(1, 1), (400, 2), (320, 16), (569, 9)])   # 5,120 and 5,121 rays: the rule's line
+@pytest.mark.parametrize("fmt", [rr.RR_NODES_BINARY, rr.RR_NODES_WIDE8])
+@pytest.mark.parametrize("cut", [0.0, 1e-7])   # visibility after and before the shading
+def test_few_lanes_equal_whole_warps(tiny_scene, n_az, rays, fmt, cut):
+    """Small scans hand their rays to 8 lanes of each query warp (64-thread
+    blocks); with blocks of 128 every warp is whole: the same queries, the same
+    image up to the rounding of the bin sums."""
+    _, pz, base, h = tiny_scene
+    p = scenes.sensor(**{**base, "n_azimuth": n_az, "rays_per_beam": rays, "min_energy": cut, "elevation": 0.1})
+    saved = rr.rr_batch_config_get(h)
+    try:
+        got = []
+        for block, split in ((128, 1), (64, 1), (64, 3)):
+            rr.rr_batch_config_set(h, node_format=fmt, trace_block=block, split_streams=split)
+            rr.rr_scene_stats(h, reset=True)
+            img = alone(h, pz, p)
+            st = rr.rr_scene_stats(h, reset=True)
+            got.append((img, st["closest_queries"], st["anyhit_queries"]))
+        for img, closest, anyhit in got[1:]:
+            assert (closest, anyhit) == got[0][1:]
+            assert_close(img, got[0][0], "few lanes")
+    finally:
+        rr.rr_batch_config_set(h, **saved)
