@@ -462,7 +462,8 @@ __device__ __forceinline__ void step_wide_node(Trav& s, uint2* stack, const Scan
   }
   const uint32_t oct = s.oct, slot = (__ffs(bits) - 1u) ^ oct;
   bits &= bits - 1u;   // the lowest bit is a pending child's
-  const uint32_t node = min(base + __popc((bits >> 8) & ((1u << slot) - 1u)), a.node_cap - 1u);
+  const uint32_t at = base + __popc((bits >> 8) & ((1u << slot) - 1u)), node = min(at, a.node_cap - 1u);
+  if (at >= a.node_cap) atomicOr(&a.ctr->error, kErrBvh);   // no build that reports success gets here
   if (bits & 0xFFu) stack[s.sp] = make_uint2(base, bits);
   s.sp += (bits & 0xFFu) ? 1 : 0;
   if (count) ++n_nodes;
