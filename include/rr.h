@@ -378,7 +378,9 @@ int rr_scan_batch_async(rr_scene* scene, uint32_t n, const rr_pose* poses, const
    use_graph            1: each launch sequence is captured once in a CUDA
                         graph and replayed while its arguments stay the same
    node_format          RR_NODES_BINARY (default): traverse the binary LBVH,
-                        its child boxes on a 16-bit grid over the scene;
+                        its child boxes on a 16-bit grid over the scene
+                        (as floats where a few far or huge triangles make
+                        that grid coarse beside the others);
                         RR_NODES_WIDE8: the 8-wide BVH with 8-bit child boxes
                         on a grid per node.  Both give the same closest hit
                         for every query (the boxes are rounded outward).

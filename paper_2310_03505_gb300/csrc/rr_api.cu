@@ -294,12 +294,25 @@ void ctx_free(ExecCtx* x) {
 
 using namespace rr_host;
 
+// what a finished build says of its grid (kCoarse), for the next one; true if that changes the nodes' form
+static bool note_coarse(rr_scene* s, const uint32_t* misc) {
+  const uint32_t coarse = misc[rr::kFrameWord + 3] != 0u ? 1u : 0u;
+  if (coarse == s->main.h_ctr->coarse) return false;
+  s->main.h_ctr->coarse = coarse;
+  if (cudaMemcpy(&s->main.d_ctr->coarse, &coarse, sizeof coarse, cudaMemcpyHostToDevice) != cudaSuccess)
+    cudaGetLastError();
+  return true;
+}
+
 int rr_host::rebuild_bvh(rr_scene* s, cudaStream_t st) {
   if (s->nt == 0) return RR_OK;
-  RR_CHECK_CUDA(build_lbvh(s, st, true), "rebuilding the BVH");
-  uint32_t misc[8];
-  RR_CHECK_CUDA(cudaMemcpyAsync(misc, s->d_misc, sizeof misc, cudaMemcpyDeviceToHost, st), "reading the build status");
-  RR_CHECK_CUDA(cudaStreamSynchronize(st), "rebuilding the BVH");
+  uint32_t misc[rr::kMiscWords];
+  for (int pass = 0; pass < 2; ++pass) {   // again if the nodes' form has to change
+    RR_CHECK_CUDA(build_lbvh(s, st, true), "rebuilding the BVH");
+    RR_CHECK_CUDA(cudaMemcpyAsync(misc, s->d_misc, sizeof misc, cudaMemcpyDeviceToHost, st), "reading the build status");
+    RR_CHECK_CUDA(cudaStreamSynchronize(st), "rebuilding the BVH");
+    if (misc[6] || !note_coarse(s, misc)) break;
+  }
   if (misc[6] & rr::kErrTopBuild) return fail(RR_ERR_CUDA, "the SAH top of the BVH could not be built");
   if (misc[6]) return fail(RR_ERR_INVALID_ARG, "the scene's vertices are invalid");
   s->depth = misc[7];
@@ -314,6 +327,7 @@ __global__ void k_fold_build_status(const uint32_t* misc, const uint32_t* wctr, 
   if (misc[6] & ~rr::kErrTopBuild) e |= rr::kErrBadVertex;
   if ((misc[6] & rr::kErrTopBuild) || wctr[4]) e |= rr::kErrBvh;
   if (e) atomicOr(&ctr->error, e);
+  ctr->coarse = misc[rr::kFrameWord + 3] != 0u ? 1u : 0u;
 }
 
 extern "C" {
@@ -363,7 +377,7 @@ int rr_scene_destroy(rr_scene* s) {
   if (!s) return RR_OK;
   cudaDeviceSynchronize();
   void* ptrs[] = {s->d_vtx, s->d_idx, s->d_mat_id, s->d_raw_mats, s->d_mats, s->d_lut, s->d_lut_cells,
-                  s->d_tri, s->d_nodes, s->d_centroid, s->d_keys[0], s->d_keys[1], s->d_vals[0], s->d_vals[1],
+                  s->d_tri, s->d_nodes, s->d_far, s->d_centroid, s->d_keys[0], s->d_keys[1], s->d_vals[0], s->d_vals[1],
                   s->d_hist, s->d_parent, s->d_child, s->d_nbox, s->d_visit, s->d_misc,
                   s->d_cut, s->d_wnodes, s->d_wtri, s->d_wsrc, s->d_wrec, s->d_wctr, s->d_lobe_kind,
                   s->d_lobe_samples, s->d_range, s->d_cl_at, s->d_cl_bsum, s->d_cl_rec,
@@ -480,7 +494,7 @@ int rr_scene_create(const float* vertices, uint32_t n_vertices, const uint32_t* 
   cudaEventDestroy(e1);
   s->build_ms = ms;
   if (n_triangles) {
-    uint32_t misc[8];
+    uint32_t misc[rr::kMiscWords];
     e = cudaMemcpy(misc, s->d_misc, sizeof misc, cudaMemcpyDeviceToHost);
     if (e != cudaSuccess) return bail(cuda_fail(e, "reading the build status"));
     if (misc[6] & 1u) return bail(fail(RR_ERR_INVALID_ARG, "a triangle references a vertex index >= n_vertices"));
@@ -490,6 +504,8 @@ int rr_scene_create(const float* vertices, uint32_t n_vertices, const uint32_t* 
     s->depth = misc[7];
     if (s->depth > (uint32_t)rr::kStack)
       return bail(fail(RR_ERR_CAPACITY, "BVH depth " + std::to_string(s->depth) + " exceeds the traversal stack"));
+    if (note_coarse(s, misc))
+      if (int rc = rebuild_bvh(s, st)) return bail(rc);
   }
   *out = s;
   return RR_OK;

@@ -466,6 +466,7 @@ int batch_enqueue(rr_scene* s, ExecCtx* x, const rr_pose* poses, const rr_sensor
   a.tri = wide ? s->d_wtri : s->d_tri;
   a.tri_copy = 3 * (size_t)s->nt;
   a.nodes = wide ? reinterpret_cast<const uint4*>(s->d_wnodes) : s->d_nodes;
+  a.far = !wide && s->exact_nodes ? s->d_far : nullptr;
   a.frame = reinterpret_cast<const float4*>(s->d_misc + rr::kFrameWord);
   a.mats = s->d_mats;
   a.lut = s->d_lut;

@@ -15,8 +15,9 @@
 //
 // The hierarchy is a binary BVH with one triangle per leaf.  Internal node i
 // is stored in 32 bytes: both child boxes rounded outward to a 16-bit grid
-// over the scene, and the child references (layout: kNodeWords); the float
-// boxes stay in nbox.
+// over the scene, and the child references (layout: kNodeWords; where that
+// grid is too coarse, in 64 bytes with float boxes); the float boxes stay in
+// nbox.
 // Leaves are the triangles in sorted order: tri[3j..3j+2] = v0, v1, v2 with
 // v0.w = original triangle id, v1.w = material id (bit patterns).
 #include <algorithm>
@@ -64,11 +65,21 @@ __device__ __forceinline__ void st_release_u32(uint32_t* p, uint32_t v) {
 // a1: validation, centroids and centroid bounds
 // misc[0..2] = ~encoded min xyz of the centroids, misc[3..5] = encoded max
 // xyz, misc[6] = error, misc[8..13] = the same bounds of the vertices (each a
-// maximum, so that all start from zero)
+// maximum, so that all start from zero), misc[14..15] = sum over the triangles
+// with an extent of the float bits of their largest extent, without the last
+// 15 (piecewise linear in its logarithm, so the mean is near the geometric
+// one and a few huge triangles do not move it), misc[16] = their count
 __global__ void k_ingest(const float* __restrict__ vtx, const uint32_t* __restrict__ idx,
                          const uint16_t* __restrict__ mat_id, uint32_t nv, uint32_t nt, uint32_t nm,
                          float4* __restrict__ centroid, uint32_t* __restrict__ misc) {
   __shared__ float s_lo[6][32], s_hi[6][32];
+  __shared__ unsigned long long s_size;
+  __shared__ uint32_t s_sized;
+  if (threadIdx.x == 0) {
+    s_size = 0ull;
+    s_sized = 0u;
+  }
+  uint32_t size = 0u, sized = 0u;   // a thread has at most some 3,500 of 2^30 triangles: size < 2^32
   float lo[6], hi[6];   // centroid, vertices
   for (int k = 0; k < 6; ++k) {
     lo[k] = INFINITY;
@@ -102,10 +113,16 @@ __global__ void k_ingest(const float* __restrict__ vtx, const uint32_t* __restri
         lo[3 + k] = fminf(lo[3 + k], vlo[k]);
         hi[3 + k] = fmaxf(hi[3 + k], vhi[k]);
       }
+      const float ext = fmaxf(fmaxf(vhi[0] - vlo[0], vhi[1] - vlo[1]), vhi[2] - vlo[2]);
+      size += __float_as_uint(ext) >> 15;
+      sized += ext > 0.0f ? 1u : 0u;
     }
     centroid[i] = make_float4(cen[0], cen[1], cen[2], 0.f);
   }
-  // warp then block reduction of the bounds
+  // warp then block reduction of the bounds and sizes
+  unsigned long long wsize = size;
+  for (int off = 16; off > 0; off >>= 1) wsize += __shfl_xor_sync(0xFFFFFFFFu, wsize, off);
+  sized = __reduce_add_sync(0xFFFFFFFFu, sized);
   for (int k = 0; k < 6; ++k) {
     for (int off = 16; off > 0; off >>= 1) {
       lo[k] = fminf(lo[k], __shfl_xor_sync(0xFFFFFFFFu, lo[k], off));
@@ -119,6 +136,15 @@ __global__ void k_ingest(const float* __restrict__ vtx, const uint32_t* __restri
       s_hi[k][warp] = hi[k];
     }
   __syncthreads();
+  if (lane == 0 && sized) {
+    atomicAdd(&s_size, wsize);
+    atomicAdd(&s_sized, sized);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0 && s_sized) {
+    atomicAdd(reinterpret_cast<unsigned long long*>(misc + kSizeWord), s_size);
+    atomicAdd(&misc[kSizeWord + 2], s_sized);
+  }
   if (warp == 0) {
     for (int k = 0; k < 6; ++k) {
       float l = lane < nw ? s_lo[k][lane] : INFINITY, h = lane < nw ? s_hi[k][lane] : -INFINITY;
@@ -144,6 +170,16 @@ __device__ __forceinline__ uint32_t spread3(uint32_t v) {
   return v;
 }
 
+// Grid step (of its coarser half) over the mean triangle size above which the
+// binary nodes should hold float boxes.  Scans of 400 x 200 rays over the
+// repository's scenes (their own grids: 0.004 to 0.021) with one more triangle
+// below the ground that stretches the grid, grid / float boxes in us:
+//   200k campus  0.004  895 / 980   0.067  979 / 958    0.22 1,143 / 964   2.2  2,834 / 952   22  48,370 / 955
+//   1M campus    0.012  814 / 864   0.070  869 / 864    0.21   925 / 865   0.70 1,123 / 862
+//   5M city      0.021  970 / 1,089 0.061  1,017 / 1,089 0.18 1,101 / 1,090 0.61 1,276 / 1,090
+// (the coarser the grid, the more triangles share a cell: 3 to 770 tests a query).
+constexpr float kCoarse = 0.125f;
+
 // a2: code = x9 y9 z9 x8 y8 z8 ... x0 y0 z0 of the quantised centroid
 // also counts the first sort pass's digits per tile (hist0, zeroed before)
 // and lays the grid of the binary nodes over the vertex bounds
@@ -157,6 +193,7 @@ __global__ void k_morton(const float4* __restrict__ centroid, uint32_t* __restri
     // either side for the outward rounding.  The scale is at least 2^-11 of
     // the coordinates, so that rounding the base moves no bound out of range.
     float* fr = reinterpret_cast<float*>(misc + kFrameWord);
+    float widest = 0.0f;
     for (int k = 0; k < 3; ++k) {
       float lo = dec_f(~misc[8 + k]), hi = dec_f(misc[11 + k]);
       if (!(lo <= hi)) lo = hi = 0.0f;   // no valid triangle: the build is reported as failed
@@ -165,8 +202,13 @@ __global__ void k_morton(const float4* __restrict__ centroid, uint32_t* __restri
       fr[k] = lo - 0.501f * scale;
       fr[4 + k] = scale;
       fr[8 + k] = 1.0f / scale;   // for the nodes' codes
+      widest = fmaxf(widest, scale);
     }
-    fr[3] = fr[7] = fr[11] = 0.0f;
+    const uint32_t sized = misc[kSizeWord + 2];
+    const unsigned long long size = *reinterpret_cast<const unsigned long long*>(misc + kSizeWord);
+    const float mean = sized ? __uint_as_float((uint32_t)(size / sized) << 15) : INFINITY;
+    fr[3] = 0x1p-15f * widest > kCoarse * mean ? 1.0f : 0.0f;
+    fr[7] = fr[11] = 0.0f;
   }
   const float4 c = centroid[i];
   const float cc[3] = {c.x, c.y, c.z};
@@ -569,9 +611,21 @@ __device__ __forceinline__ uint32_t grid_hi(float x, float base, float inv) {
   return ((__float_as_uint(f) + 0xFFu) >> 8) & 0xFFFFu;
 }
 
-// binary node p: boxes b0, b1 (lo xyz, hi xyz) of its children c0, c1
-__device__ __forceinline__ void write_node(uint4* __restrict__ nodes, size_t p, const float* __restrict__ frame,
-                                           const float* b0, const float* b1, uint32_t c0, uint32_t c1) {
+// binary node p: boxes b0, b1 (lo xyz, hi xyz) of its children c0, c1; far:
+// the second array of nodes with float boxes, or null for nodes on the grid
+__device__ __forceinline__ void write_node(uint4* __restrict__ nodes, uint4* __restrict__ far, size_t p,
+                                           const float* __restrict__ frame, const float* b0, const float* b1,
+                                           uint32_t c0, uint32_t c1) {
+  if (far != nullptr) {
+    const auto half = [p](uint4* q, const float* b, uint32_t r0, uint32_t r1) {
+      q += kNodeWords * p;
+      q[0] = make_uint4(__float_as_uint(b[0]), __float_as_uint(b[3]), __float_as_uint(b[1]), __float_as_uint(b[4]));
+      q[1] = make_uint4(__float_as_uint(b[2]), __float_as_uint(b[5]), r0, r1);
+    };
+    half(nodes, b0, c0, c1);
+    half(far, b1, 0u, 0u);
+    return;
+  }
   uint32_t w[6];
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
@@ -597,7 +651,7 @@ __global__ void __launch_bounds__(kRefitBlock) k_refit(uint32_t n, const uint32_
                                                        const uint32_t* __restrict__ parent,
                                                        const uint2* __restrict__ range, uint32_t* __restrict__ visit,
                                                        float* __restrict__ nbox, uint4* __restrict__ nodes,
-                                                       const float* __restrict__ frame) {
+                                                       uint4* __restrict__ far, const float* __restrict__ frame) {
   __shared__ float s_box[2][kRefitBlock][6];   // [0] the block's leaves, [1] its local internal nodes
   __shared__ uint32_t s_visit[kRefitBlock];
   const uint32_t base = blockIdx.x * kRefitBlock, end = min(base + kRefitBlock, n);
@@ -641,7 +695,7 @@ __global__ void __launch_bounds__(kRefitBlock) k_refit(uint32_t n, const uint32_
       b0[k] = first_is_own ? own[k] : sb[k];
       b1[k] = first_is_own ? sb[k] : own[k];
     }
-    write_node(nodes, p, frame, b0, b1, c0, c1);
+    write_node(nodes, far, p, frame, b0, b1, c0, c1);
     float* bp = nbox + 6 * (size_t)p;
     for (int k = 0; k < 3; ++k) {
       own[k] = fminf(b0[k], b1[k]);
@@ -835,6 +889,7 @@ struct TopArgs {
   uint32_t* ctr;          // kCtr*
   uint32_t* cb;           // [T - 1][6] centroid bounds (encoded) of the block task at each node slot
   uint4* nodes;
+  uint4* far;             // second array of binary nodes with float boxes, or null
   const float* frame;     // grid of the binary nodes
   uint32_t* child;
   uint32_t* parent;
@@ -946,7 +1001,7 @@ __device__ Split warp_best_split(const uint32_t* bins, int lane) {
 // the node of a task: child boxes (lo xyz, hi xyz) and references
 __device__ __forceinline__ void write_top_node(const TopArgs& a, uint32_t slot, const float (&bx)[2][6],
                                                const uint32_t (&ref)[2]) {
-  write_node(a.nodes, slot, a.frame, bx[0], bx[1], ref[0], ref[1]);
+  write_node(a.nodes, a.far, slot, a.frame, bx[0], bx[1], ref[0], ref[1]);
   a.child[2 * slot] = ref[0];
   a.child[2 * slot + 1] = ref[1];
   for (int side = 0; side < 2; ++side) a.parent[node_slot(ref[side], a.n)] = slot;
@@ -2067,6 +2122,7 @@ static cudaError_t build_sah_top(rr_scene* s, cudaStream_t st) {
   a.ctr = s->d_top_ctr;
   a.cb = s->d_top_cb;
   a.nodes = s->d_nodes;
+  a.far = s->exact_nodes ? s->d_far : nullptr;
   a.frame = reinterpret_cast<const float*>(s->d_misc + kFrameWord);
   a.child = s->d_child;
   a.parent = s->d_parent;
@@ -2089,7 +2145,15 @@ static cudaError_t build_sah_top(rr_scene* s, cudaStream_t st) {
 
 cudaError_t build_lbvh(rr_scene* s, cudaStream_t st, bool with_depth) {
   const uint32_t n = s->nt;
-  // bounds, error and depth start from zero
+  // the form of the binary nodes, as the last build that the host has heard of
+  // asks for (kCoarse); without memory for it, the grid
+  if (s->main.h_ctr->coarse && !s->d_far && n > 1) {
+    const size_t bytes = (size_t)(n - 1) * kNodeWords * sizeof(uint4);
+    if (dev_malloc(&s->d_far, bytes) == cudaSuccess) s->scene_bytes += bytes;
+    else cudaGetLastError();
+  }
+  s->exact_nodes = s->main.h_ctr->coarse && s->d_far;
+  // bounds, error, depth and sizes start from zero
   RR_TRY(cudaMemsetAsync(s->d_misc, 0, kFrameWord * sizeof(uint32_t), st));
   if (n == 0) return cudaSuccess;
   const int B = 256;
@@ -2137,6 +2201,7 @@ cudaError_t build_lbvh(rr_scene* s, cudaStream_t st, bool with_depth) {
     RR_TRY(cudaGetLastError());
     k_refit<<<(n + kRefitBlock - 1) / kRefitBlock, kRefitBlock, 0, st>>>(n, s->d_child, s->d_parent, s->d_range,
                                                                            s->d_visit, s->d_nbox, s->d_nodes,
+                                                                           s->exact_nodes ? s->d_far : nullptr,
                                                                            reinterpret_cast<const float*>(s->d_misc + kFrameWord));
     RR_TRY(cudaGetLastError());
     if (sah_top) RR_TRY(build_sah_top(s, st));

@@ -93,7 +93,9 @@ struct rr_scene {
   std::vector<uint32_t> raw_flags; // rr_material.flags of every material
   float* d_lobe_samples = nullptr; // [M][kLobeSamples] tabulated lobes (allocated on first use)
   float4* d_tri = nullptr;         // [3][T][3] sorted leaves in three rotated copies, then [T] unit normals
-  uint4* d_nodes = nullptr;        // [T-1][kNodeWords] quantised binary nodes
+  uint4* d_nodes = nullptr;        // [T-1][kNodeWords] binary nodes
+  uint4* d_far = nullptr;          // the same for child 1's float boxes (allocated with the first such build)
+  bool exact_nodes = false;        // the binary nodes hold float boxes
   // 8-wide quantised BVH (collapsed from the binary one at every build)
   uint32_t wcap = 0;               // wide node capacity (T - 1, at least 1)
   uint32_t wide_epoch = 0;         // build counter tagging the published work items
@@ -113,7 +115,7 @@ struct rr_scene {
   uint32_t* d_child = nullptr;     // [T-1][2]
   float* d_nbox = nullptr;         // [2T-1][6]
   uint32_t* d_visit = nullptr;     // [T-1]
-  uint32_t* d_misc = nullptr;      // [kMiscWords]: bounds (encoded), error bits, depth, node grid
+  uint32_t* d_misc = nullptr;      // [kMiscWords]: bounds (encoded), error bits, depth, sizes, node grid
   uint2* d_range = nullptr;        // [T-1] leaf range (first, last) of every internal node
   // SAH top over the LBVH's subtrees (allocated with the first such build)
   uint32_t* d_cl_at = nullptr;     // [T] cluster root reference at the cluster's first leaf, else kNone

@@ -94,7 +94,7 @@ struct ScanCounters {
   uint32_t vis_ticket[RR_MAX_BOUNCES];
   uint32_t need_rays, need_recs;           // largest request seen (overflow report)
   uint32_t error;                          // sticky kErr* bits
-  uint32_t pad;
+  uint32_t coarse;                         // the scene's grid is too coarse (kCoarse), as of its last build
   unsigned long long stat_closest, stat_anyhit, stat_returns, stat_scans;
   unsigned long long stat_nodes, stat_tris;
   unsigned long long stat_nodes_any, stat_tris_any;
@@ -124,10 +124,19 @@ constexpr int kWideNodeWords = 5;
 // closest-hit query pays for is the fetch (2 x 128 bits against 4, and half
 // the L1 and L2 footprint), and one byte permutation per plane picks the near
 // or far plane and decodes it, where the float form needed a min and a max.
+//
+// One grid serves the whole scene, so its step grows with the farthest vertex
+// while the boxes do not.  Where it is coarse beside the triangles (kCoarse)
+// the nodes hold the float boxes instead, from the next build after the host
+// has heard of it (build_lbvh): child 0's in the node, child 1's in the same
+// place of a second array, each as (lo x, hi x, lo y, hi y) (lo z, hi z,
+// child0, child1), the references with child 0 only.
 constexpr int kNodeWords = 2;
-// The grid of a scene's binary nodes, three float4: (base x, y, z, 0), (scale x, y, z, 0), (1 / scale, 0)
-constexpr int kFrameWord = 16;        // its place in the build status words (rr_scene::d_misc)
-constexpr int kMiscWords = 28;        // 0..5 centroid bounds, 6 error bits, 7 depth, 8..13 vertex bounds, 16..27 the frame
+// The grid of a scene's binary nodes, three float4: (base x, y, z, f), (scale x, y, z, 0), (1 / scale, 0),
+// f: 1 where it is too coarse
+constexpr int kFrameWord = 20;        // its place in the build status words (rr_scene::d_misc)
+constexpr int kSizeWord = 14;         // sum (64 bits) and count of the triangles' sizes (k_ingest)
+constexpr int kMiscWords = 32;        // 0..5 centroid bounds, 6 error bits, 7 depth, 8..13 vertex bounds, 14..16 sizes, 20..31 the frame
 
 // Return record key: global image column (scan's first column + azimuth)
 // and range bin.  Records of one bounce are in column order.
@@ -166,7 +175,8 @@ struct ScanArgs {
                              // (unit geometric normal, material bits) at tri + 3 tri_copy
   size_t tri_copy;           // float4s from one rotated copy to the next (3 T)
   const uint4* nodes;        // binary: [T-1][kNodeWords], wide: [.][kWideNodeWords]
-  const float4* frame;       // [2] grid of the binary nodes' boxes
+  const uint4* far;          // binary nodes with float boxes: [T-1][kNodeWords], else null
+  const float4* frame;       // [3] grid of the binary nodes' boxes
   const MatDev* mats;
   const float4* lut;         // [M][kLutCells + 1]: (G(x_k), Gc(x_k), cos^C(x_k), 0)
   uint32_t n_tris, n_mats;

@@ -240,7 +240,7 @@ __device__ __forceinline__ float2 fma2(float a, float b, float m, unsigned long 
 // lexicographically smallest.  Any hit: the first t_min < t < t_best.  The
 // leaf `skip` (the one the ray starts on) is never reported.
 struct Trav {
-  float3 c0, c1;        // slab offsets of the near / far planes (trav_begin)
+  float3 c0, c1;        // slab offsets of the near / far planes (float boxes: the lower / upper ones; trav_begin)
   WoopRay w;            // the watertight-test frame
   float3 id;            // 1 / direction, zero components replaced by +-1e-30; binary nodes: times the grid scale
   uint3 sel;            // binary: byte selectors that decode the near plane of a box word, per axis
@@ -254,13 +254,14 @@ struct Trav {
   int sp;                                     // next free stack entry (binary: its byte offset)
 };
 
+// exact: binary nodes with float boxes
 __device__ __forceinline__ void trav_begin(Trav& s, const ScanArgs& a, float3 o, float3 d, float t_min, float t_best,
-                                           uint32_t skip, bool wide) {
+                                           uint32_t skip, bool wide, bool exact) {
   s.w = make_woop(o, d);
   const float3 dn = make_float3(fabsf(d.x) > 1e-30f ? d.x : copysignf(1e-30f, d.x),
                                 fabsf(d.y) > 1e-30f ? d.y : copysignf(1e-30f, d.y),
                                 fabsf(d.z) > 1e-30f ? d.z : copysignf(1e-30f, d.z));
-  if (wide) {
+  if (wide || exact) {
     s.id = make_float3(1.0f / dn.x, 1.0f / dn.y, 1.0f / dn.z);
     // Slab test with one fma per plane: plane b is reached at t = fma(b, id, c)
     // with c = -(o id) -+ eps, where the robust form (b - o) id needs two
@@ -272,7 +273,12 @@ __device__ __forceinline__ void trav_begin(Trav& s, const ScanArgs& a, float3 o,
     // slab test (1 + 2 gamma_3, Ize 2013) at the node.  So a box the robust
     // test accepts is accepted here too.
     const float ox = __fmul_rn(o.x, s.id.x), oy = __fmul_rn(o.y, s.id.y), oz = __fmul_rn(o.z, s.id.z);
-    const float ex = 0x1p-22f * fabsf(ox), ey = 0x1p-22f * fabsf(oy), ez = 0x1p-22f * fabsf(oz);
+    float ex = 0x1p-22f * fabsf(ox), ey = 0x1p-22f * fabsf(oy), ez = 0x1p-22f * fabsf(oz);
+    if (exact) {   // the lower plane is the near one for a positive direction component
+      ex = copysignf(ex, s.id.x);
+      ey = copysignf(ey, s.id.y);
+      ez = copysignf(ez, s.id.z);
+    }
     s.c0 = make_float3(-ox - ex, -oy - ey, -oz - ez);
     s.c1 = make_float3(-ox + ex, -oy + ey, -oz + ez);
   } else {
@@ -407,6 +413,35 @@ __device__ __forceinline__ void step_inner(Trav& s, uint32_t* stack, const ScanA
   if (both) bin_entry(stack, s.sp) = far;
   s.sp += both ? 4 : (any ? 0 : -4);
   s.node = any ? near : top;
+}
+
+// Binary BVH with float boxes (kNodeWords): the same visit
+__device__ __forceinline__ void step_inner_exact(Trav& s, uint32_t* stack, const ScanArgs& a, uint32_t& n_nodes,
+                                                 bool count) {
+  if (count) ++n_nodes;
+  ++s.visits;
+  const uint32_t top = bin_entry(stack, s.sp - 4);
+  const size_t at = kNodeWords * (size_t)s.node;
+  const float4* n0 = reinterpret_cast<const float4*>(a.nodes + at);
+  const float4* n1 = reinterpret_cast<const float4*>(a.far + at);
+  const float4 x0 = __ldg(n0), x1 = __ldg(n1), z0 = __ldg(n0 + 1), z1 = __ldg(n1 + 1);
+  const float3 id = s.id, cl = s.c0, ch = s.c1;
+  float lo[2], hi[2];
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const float4 xy = k ? x1 : x0, z = k ? z1 : z0;
+    const float tx0 = fmaf(xy.x, id.x, cl.x), tx1 = fmaf(xy.y, id.x, ch.x);
+    const float ty0 = fmaf(xy.z, id.y, cl.y), ty1 = fmaf(xy.w, id.y, ch.y);
+    const float tz0 = fmaf(z.x, id.z, cl.z), tz1 = fmaf(z.y, id.z, ch.z);
+    lo[k] = fmaxf(max3(fminf(tx0, tx1), fminf(ty0, ty1), fminf(tz0, tz1)), s.t_min);
+    hi[k] = fminf(min3(fmaxf(tx0, tx1), fmaxf(ty0, ty1), fmaxf(tz0, tz1)) * kBoxInflate, s.t_best);
+  }
+  const bool h0 = lo[0] <= hi[0], h1 = lo[1] <= hi[1], both = h0 && h1, any = h0 || h1;
+  const bool first0 = !h1 || (h0 && lo[0] <= lo[1]);
+  const uint32_t c0 = __float_as_uint(z0.z), c1 = __float_as_uint(z0.w);
+  if (both) bin_entry(stack, s.sp) = first0 ? c1 : c0;
+  s.sp += both ? 4 : (any ? 0 : -4);
+  s.node = any ? (first0 ? c0 : c1) : top;
 }
 
 // Binary BVH: one leaf
@@ -609,7 +644,9 @@ constexpr int kQueryThreads = 1152;
 // the kernels of the scans that ask for them
 // kSpread: only a.lanes lanes of a warp take queries (small launch sequences);
 // apart, because the whole-warp kernels lose 1 % to the extra operands.
-template <bool kAny, int kBlock, bool kWide, bool kCount, bool kSpread>
+// kExact: binary nodes with float boxes; a kernel of its own, because a choice
+// inside costs the scans over the grid 2 to 3 % in registers.
+template <bool kAny, int kBlock, bool kWide, bool kCount, bool kSpread, bool kExact>
 __global__ void __launch_bounds__(kBlock, kWide ? 0 : kQueryThreads / kBlock) k_query(ScanArgs a, uint32_t bounce) {
   typedef typename std::conditional<kWide, uint2, uint32_t>::type StackEntry;
   ScanCounters* C = a.ctr;
@@ -681,7 +718,7 @@ __global__ void __launch_bounds__(kBlock, kWide ? 0 : kQueryThreads / kBlock) k_
           const float3 v = f3(__ldg(&sd->pos_rmax)) - p;
           const float dist = length(v);
           dir = (1.0f / dist) * v;
-          trav_begin(s, a, p, dir, __ldg(&sd->phys.x), dist, __float_as_uint(pl.w), kWide);
+          trav_begin(s, a, p, dir, __ldg(&sd->phys.x), dist, __float_as_uint(pl.w), kWide, kExact);
         } else if (kAny) {
           const uint2 jb = jobs[job];
           ray_i = jb.x;
@@ -695,7 +732,7 @@ __global__ void __launch_bounds__(kBlock, kWide ? 0 : kQueryThreads / kBlock) k_
           const float3 v = f3(__ldg(&sd->pos_rmax)) - p;
           const float dist = length(v);
           dir = (1.0f / dist) * v;
-          trav_begin(s, a, p, dir, __ldg(&sd->phys.x), dist, h.leaf, kWide);
+          trav_begin(s, a, p, dir, __ldg(&sd->phys.x), dist, h.leaf, kWide, kExact);
         } else {
           ray_i = perm ? perm[job] : job;
           if (ray_i >= n) ray_i = job;   // only after a failed shading pass (the scan reports it)
@@ -705,7 +742,7 @@ __global__ void __launch_bounds__(kBlock, kWide ? 0 : kQueryThreads / kBlock) k_
           const float n_cur = sm.y == kAir ? 1.0f : __ldg(&a.mats[sm.y].n);
           // past t_lim no return can reach the image
           dir = f3(ray.d_E);
-          trav_begin(s, a, f3(ray.o_L), dir, phys.x, (phys.w - ray.o_L.w) / n_cur, ray.meta.x, kWide);
+          trav_begin(s, a, f3(ray.o_L), dir, phys.x, (phys.w - ray.o_L.w) / n_cur, ray.meta.x, kWide, kExact);
         }
         if (kWide) {
           reinterpret_cast<uint2*>(stack)[0] = make_uint2(0u, 0u);
@@ -745,7 +782,10 @@ __global__ void __launch_bounds__(kBlock, kWide ? 0 : kQueryThreads / kBlock) k_
         for (int u = 0; u < kSteps && s.node != kNone; u += kNodeSteps) {
 #pragma unroll
           for (int v = 0; v < kNodeSteps; ++v)
-            if (!(s.node & kLeafBit)) step_inner(s, st, a, n_nodes, count);   // kNone carries the leaf bit
+            if (!(s.node & kLeafBit)) {   // kNone carries the leaf bit
+              if (kExact) step_inner_exact(s, st, a, n_nodes, count);
+              else step_inner(s, st, a, n_nodes, count);
+            }
           if ((s.node & kLeafBit) && s.node != kNone) step_leaf<kAny>(s, st, a, n_tris, count);
           if (s.sp > 4 * (1 + kStack)) {   // a tree deeper than the stack: the scan reports it
             atomicOr(&a.ctr->error, kErrStack);
@@ -1384,7 +1424,7 @@ static int block_index(uint32_t block) { return block <= 64u ? 0 : (block <= 128
 
 template <bool kAny, int kBlock, bool kWide>
 static void occ_of(int* out) {
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, k_query<kAny, kBlock, kWide, false, false>, kBlock, 0);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, k_query<kAny, kBlock, kWide, false, false, false>, kBlock, 0);
   if (*out < 1) *out = 1;
 }
 
@@ -1429,23 +1469,23 @@ cudaError_t launch_raygen(const ScanArgs& a, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-template <bool kAny, bool kWide, bool kCount>
+template <bool kAny, bool kWide, bool kCount, bool kExact>
 static void query_launch_c(const ScanArgs& a, uint32_t bounce, int bi, int grid, cudaStream_t st) {
   if (bi == 0) {
-    if (a.lanes < 32u && !kCount) k_query<kAny, 64, kWide, false, true><<<grid, 64, 0, st>>>(a, bounce);
-    else k_query<kAny, 64, kWide, kCount, false><<<grid, 64, 0, st>>>(a, bounce);
+    if (a.lanes < 32u && !kCount) k_query<kAny, 64, kWide, false, true, kExact><<<grid, 64, 0, st>>>(a, bounce);
+    else k_query<kAny, 64, kWide, kCount, false, kExact><<<grid, 64, 0, st>>>(a, bounce);
   } else if (bi == 1) {
-    k_query<kAny, 128, kWide, kCount, false><<<grid, 128, 0, st>>>(a, bounce);
+    k_query<kAny, 128, kWide, kCount, false, kExact><<<grid, 128, 0, st>>>(a, bounce);
   } else {
-    k_query<kAny, 256, kWide, kCount, false><<<grid, 256, 0, st>>>(a, bounce);
+    k_query<kAny, 256, kWide, kCount, false, kExact><<<grid, 256, 0, st>>>(a, bounce);
   }
 }
-template <bool kAny, bool kWide>
+template <bool kAny, bool kWide, bool kExact>
 static void query_launch(const ScanArgs& a, uint32_t bounce, int bi, int grid, cudaStream_t st) {
   // a counting kernel may hold more registers: its blocks beyond the
   // residency start later and find no work left
-  if (a.any_flags & RR_COUNT_TRAVERSAL) query_launch_c<kAny, kWide, true>(a, bounce, bi, grid, st);
-  else query_launch_c<kAny, kWide, false>(a, bounce, bi, grid, st);
+  if (a.any_flags & RR_COUNT_TRAVERSAL) query_launch_c<kAny, kWide, true, kExact>(a, bounce, bi, grid, st);
+  else query_launch_c<kAny, kWide, false, kExact>(a, bounce, bi, grid, st);
 }
 
 cudaError_t launch_query(const ScanArgs& a, uint32_t bounce, bool any, const LaunchCfg& c, cudaStream_t st) {
@@ -1458,11 +1498,14 @@ cudaError_t launch_query(const ScanArgs& a, uint32_t bounce, bool any, const Lau
   const uint64_t warps = (((uint64_t)a.n_rays0 << bounce) + a.lanes - 1) / a.lanes, per_block = 2u << bi;
   const int grid = (int)std::max<uint64_t>(1, std::min<uint64_t>((uint64_t)g_num_sms * per_sm, (warps + per_block - 1) / per_block));
   if (wide) {
-    if (any) query_launch<true, true>(a, bounce, bi, grid, st);
-    else query_launch<false, true>(a, bounce, bi, grid, st);
+    if (any) query_launch<true, true, false>(a, bounce, bi, grid, st);
+    else query_launch<false, true, false>(a, bounce, bi, grid, st);
+  } else if (a.far) {
+    if (any) query_launch<true, false, true>(a, bounce, bi, grid, st);
+    else query_launch<false, false, true>(a, bounce, bi, grid, st);
   } else {
-    if (any) query_launch<true, false>(a, bounce, bi, grid, st);
-    else query_launch<false, false>(a, bounce, bi, grid, st);
+    if (any) query_launch<true, false, false>(a, bounce, bi, grid, st);
+    else query_launch<false, false, false>(a, bounce, bi, grid, st);
   }
   return cudaGetLastError();
 }
