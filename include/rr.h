@@ -383,7 +383,10 @@ int rr_scan_batch_async(rr_scene* scene, uint32_t n, const rr_pose* poses, const
                         that grid coarse beside the others);
                         RR_NODES_WIDE8: the 8-wide BVH with 8-bit child boxes
                         on a grid per node.  Both give the same closest hit
-                        for every query (the boxes are rounded outward).
+                        (the boxes are rounded outward); where a ray meets two
+                        triangles at one distance up to rounding (an edge they
+                        share, overlap in one plane), either may report the
+                        other of the two.
    refill_threshold     the query kernels keep their lanes busy by handing a
                         warp's idle lanes new queries once at least this many
                         of its 32 lanes are idle (1..32; 0 = 16).  Scans of at
@@ -408,7 +411,8 @@ int rr_scan_batch_async(rr_scene* scene, uint32_t n, const rr_pose* poses, const
                         RR_BVH_LBVH: the LBVH alone.  Every build of the
                         scene (creation, rr_scene_update_vertices) uses it;
                         setting a different value rebuilds the BVH (blocking).
-                        Both give the same closest hit for every query; the
+                        Both give the same closest hit, up to the same choice
+                        between triangles at one distance; the
                         SAH top needs fewer node visits.
    query_order          order in which the closest-hit queries of bounces >= 1
                         are handed to the query kernel: RR_ORDER_QUEUE (the

@@ -24,8 +24,9 @@
 // them.
 //
 // The static path always traverses the binary BVH, which every build makes:
-// both node formats give the same closest hit for every query, and the
-// binary nodes never need the lazy collapse of the 8-wide BVH.
+// both node formats find the same closest hits (up to the choice between
+// triangles at one distance), and the binary nodes never need the lazy
+// collapse of the 8-wide BVH.
 #include <cuda_runtime.h>
 
 #include <mutex>

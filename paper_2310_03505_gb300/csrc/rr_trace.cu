@@ -165,16 +165,19 @@ __device__ __forceinline__ float woop_hit(const WoopRay& w, float3 v0, float3 v1
 }
 
 // Where two triangles share an edge, the test above takes the ray that meets it
-// for both, at distances that differ in their last bits, and takes rays a
-// rounding error beside an outer edge.  Which of these count is decided by the
-// triangle's own float box, not by the coarser boxes of the nodes: a hit next
-// to an edge stands only if the robust slab test of that box (planes at
-// fma(b, 1/d, -o/d) moved apart by 4 u |o/d|, far planes inflated by 1 + 2
-// gamma_3) accepts the ray up to the best hit so far.  So the same one of two
-// such triangles is found whatever the nodes' grid (one path in some 10^8
-// queries turned at a building's edge without it; 4 % of a scan).  Apart from
-// the loop, for its registers: inlined it costs 2 % more.  v, o and d in the
-// frame of the triangle copy.
+// for both, at distances that differ in their last bits.  Either is a right
+// answer; nodes with float boxes report the one whose hit is found first
+// unless the other's box begins before that hit, because the slab test culls
+// it.  The coarser boxes of the grid would let the other one win, and a path
+// at a building's corner turn the other way (one in some 10^8 queries).  So
+// over the grid a hit next to an edge stands only if that slab test of the
+// triangle's own float box (planes at fma(b, 1/d, -o/d) moved apart by 4 u
+// |o/d|, far planes inflated by 1 + 2 gamma_3) accepts the ray up to the best
+// hit so far.  That depends on the order of the visits, so it makes the two
+// forms agree in nearly all of these cases, not in all; without the best hit
+// in the test it would decide none of them.  4 % of a scan.  Apart from the
+// loop, for its registers: inlined it costs 2 % more.  v, o and d in the frame
+// of the triangle copy.
 constexpr float kBoxInflate = 1.00000036f;   // 1 + 2 gamma_3 (Ize 2013)
 __device__ __noinline__ bool edge_hit_stands(float3 v0, float3 v1, float3 v2, float3 o, float3 d, float t_min,
                                              float t_best) {
@@ -237,8 +240,10 @@ __device__ __forceinline__ float2 fma2(float a, float b, float m, unsigned long 
 // lanes of its warp go on.
 //
 // Closest hit: t_min < t < t_best on entry, (t, original id)
-// lexicographically smallest.  Any hit: the first t_min < t < t_best.  The
-// leaf `skip` (the one the ray starts on) is never reported.
+// lexicographically smallest of the triangles tested; of triangles whose t
+// agree up to rounding (a shared edge, overlap in one plane) the boxes may
+// leave out all but one, the node format and build decide which.  Any hit:
+// the first t_min < t < t_best.  The leaf `skip` (the one the ray starts on) is never reported.
 struct Trav {
   float3 c0, c1;        // slab offsets of the near / far planes (float boxes: the lower / upper ones; trav_begin)
   WoopRay w;            // the watertight-test frame
@@ -467,7 +472,7 @@ __device__ __forceinline__ void step_leaf(Trav& s, uint32_t* stack, const ScanAr
 // lowest entry is empty and ends the query.  Slot boxes (see kWideNodeWords)
 // contain the box of the binary node they stand for, and both node formats
 // take a conservative slab test, so a query reaches every triangle it can hit
-// in either BVH and finds the same closest hit.
+// in either BVH and finds the same closest hit (up to rounding, see Trav).
 //
 // Slab test: byte q of a plane word becomes the float F = 1 + q 2^-15 (bits
 // 0x3F80qq00), and the plane P + q s is reached at t = fma(F, g, c) with
