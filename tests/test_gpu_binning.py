@@ -80,3 +80,36 @@ def test_host_buffers_and_edge_cases(rrlib):
         run(np.array([1, 0], np.uint32), np.array([0, 0], np.uint32), np.ones(2, np.float32), 2, 4, device=False)
     with pytest.raises(rr.RRError):
         run(np.array([0, 5], np.uint32), np.array([0, 0], np.uint32), np.ones(2, np.float32), 2, 4, device=False)
+
+
+def test_calls_from_many_threads(rrlib):
+    """24 threads on streams of their own, more than the library has setup
+    blocks to hand out (16): every image is its own call's, device and host
+    buffers, refused calls between them."""
+    import threading
+
+    import torch
+    n_columns, n_bins, calls = 40, 300, 6
+    data = [returns(np.random.default_rng(100 + i), 3000 + 200 * i, n_columns, n_bins) for i in range(24)]
+    refs = [orc.bin_returns(*d, n_columns, n_bins) for d in data]
+    wrong, start = [], threading.Barrier(len(data))
+
+    def work(i):
+        try:
+            with torch.cuda.stream(torch.cuda.Stream()):
+                start.wait()
+                for k in range(calls):
+                    got = run(*data[i], n_columns, n_bins, device=(i + k) % 3 != 0)
+                    if not np.all(np.abs(got - refs[i]) <= ULPS * ulp32(refs[i])):
+                        wrong.append((i, k))
+                    with pytest.raises(rr.RRError):
+                        run(data[i][0][::-1].copy(), *data[i][1:], n_columns, n_bins)
+        except Exception as e:   # an assertion in a thread would be lost
+            wrong.append((i, repr(e)))
+
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(len(data))]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not wrong, wrong
