@@ -342,7 +342,7 @@ def batched_bench(device, stream, flush, steps: int = 3, warmup: int = 2, rank: 
         "workload": BATCHED_WORKLOAD, **batched,
         "config": {"triangles": sc.n_triangles, "n_scans": n, "n_azimuth": 400,
                    "rays_per_beam": {"min": int(min(ns)), "max": int(max(ns)), "mean": float(np.mean(ns))},
-                   "initial_rays_per_step": n0, "max_bounces": 5, "n_bins": 2000, "node_format": "wide8_q8" if tuned_cfg["node_format"] == rr.RR_NODES_WIDE8 else "binary_fp32",
+                   "initial_rays_per_step": n0, "max_bounces": 5, "n_bins": 2000, "node_format": "wide8_q8" if tuned_cfg["node_format"] == rr.RR_NODES_WIDE8 else "binary_grid16",
                    "step": "256 scans, resident BVH (no rebuild)", "bvh": bvh,
                    "l2": "flushed between steps (256 MiB write, outside the timed events)"},
         "steps": steps, "warmup": warmup,
@@ -499,7 +499,7 @@ def plain_bench(rr, device, stream, flush, sc, pz, params, steps, warmup, *, ran
             rr.rr_batch_config_set(h, query_order=rr.RR_ORDER_CELL_OCTANT if order == "cell_octant"
                                    else rr.RR_ORDER_QUEUE)
         cfg = rr.rr_batch_config_get(h)
-        nf = "wide8_q8" if cfg["node_format"] == rr.RR_NODES_WIDE8 else "binary_fp32"
+        nf = "wide8_q8" if cfg["node_format"] == rr.RR_NODES_WIDE8 else "binary_grid16"
         out.update(node_format=nf, split_streams=cfg["split_streams"] or SPLIT_DEFAULT,
                    workspace_limit=cfg["workspace_limit"],
                    query_order="cell_octant" if cfg["query_order"] == rr.RR_ORDER_CELL_OCTANT else "queue")
@@ -705,7 +705,7 @@ def main():
         import oracle.oracle as orc
         orc.build()
         value, cores, sample, t_step = oracle_reference_steps(sc, pz, params, args.steps, args.warmup)
-        nf = {"auto": "binary_fp32", "binary": "binary_fp32", "wide": "wide8_q8"}[args.node_format]
+        nf = {"auto": "binary_grid16", "binary": "binary_grid16", "wide": "wide8_q8"}[args.node_format]
         line = {"impl": "reference", "metric": METRIC, "value": value, "unit": "Mrays/s", "n_gpus": args.gpus,
                 "steps": args.steps, "warmup": args.warmup, "ms_per_step": 1e3 * t_step,
                 "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "f64",

@@ -13,7 +13,7 @@
 //           through the beam window of the material lobe (Eq. 3-5), and the
 //           reflected / refracted children.  Children and return records are
 //           compacted stably (single pass, decoupled look-back over tiles of
-//           256 rays), so every queue and every bounce's record list stays
+//           256 or 512 rays), so every queue and every bounce's record list stays
 //           in (azimuth, ray) order.
 //
 // All kernels are persistent: the grid is a multiple of the SM count and
@@ -488,7 +488,6 @@ __device__ __forceinline__ void step_leaf(Trav& s, uint32_t* stack, const ScanAr
 // before its slab fma and set the hit masks slot by slot behind branches:
 // campus scan over the wide nodes 2,447 us, 1,567 now (batch server's burst of
 // 24 requests 18.3 -> 12.1 ms); 1 / 3 visits per leaf test 1,590 / 1,658.
-template <bool kAny>
 __device__ __forceinline__ void step_wide_node(Trav& s, uint2* stack, const ScanArgs& a, uint32_t& n_nodes,
                                                bool count) {
   const uint2 top = stack[s.sp - 1];
@@ -773,7 +772,7 @@ __global__ void __launch_bounds__(kBlock, kWide ? 0 : kQueryThreads / kBlock) k_
         for (int u = 0; u < kStepsWide && s.node != kNone; u += kWideVisits) {
 #pragma unroll
           for (int v = 0; v < kWideVisits; ++v)
-            if (s.t_bits == 0u && s.node != kNone) step_wide_node<kAny>(s, st, a, n_nodes, count);
+            if (s.t_bits == 0u && s.node != kNone) step_wide_node(s, st, a, n_nodes, count);
           if (s.t_bits) step_wide_leaf<kAny>(s, a, n_tris, count);
           if (s.sp > 1 + kStack) {   // deeper than the stack: the scan reports it
             atomicOr(&a.ctr->error, kErrStack);
@@ -1122,7 +1121,7 @@ __global__ void __launch_bounds__(kBlock, kMinBlocks) k_shade(ScanArgs a, uint32
     uint32_t kmed = 0u;
     uint2 rt = make_uint2(0u, 0u), ra = rt;
     bool cand = false;           // an air-path candidate left to the visibility query (deferred visibility)
-    int vj_kid = -1, vj_rec = -1;   // its child in kid[], its record in rec[] (-1: none)
+    int vj_kid = -1, vj_rec = -1;   // its child and record among this ray's (-1: none)
     if (i < n) {
       const RayRec ray = qin[i];
       const HitRec h = a.hits[i];
@@ -1366,13 +1365,12 @@ __global__ void __launch_bounds__(kBlock, kMinBlocks) k_shade(ScanArgs a, uint32
     kid[1].d_E = make_float4(d_refr.x, d_refr.y, d_refr.z, e_refr);
     kid[0].meta = kmeta;
     kid[1].meta = make_uint4(kmeta.x, kmeta.y, kmeta.z | 1u, kmed);
-    const bool counts = a.order_key != nullptr && bounce + 1 < a.max_bounces;
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
       const uint32_t pos = kbase + (c && sp_refl ? 1u : 0u);
       if ((c ? sp_refr : sp_refl) && pos < a.ray_cap) {
         qout[pos] = kid[c];
-        if (counts) {   // order bucket of the child, counted in the block's histogram
+        if (counting) {   // order bucket of the child, counted in the block's histogram
           const uint32_t key = order_key(a, kid[c]);
           a.order_key[pos] = (uint16_t)key;
           atomicAdd(&s_hist[key], 1u);
