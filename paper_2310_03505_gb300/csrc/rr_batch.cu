@@ -381,7 +381,7 @@ static int graph_launch(rr_scene* s, ExecCtx* x, const ScanArgs& a, bool pattern
 // most of the chip without a warp while its own warps run through the union of
 // 32 rays' visits: fewer rays a warp shorten that, until the warps no longer
 // fit beside each other.  rays: those in flight together, all ranges of a
-// split scan.  Whole scans over 5 bounces, 8 / 16 / 32 lanes, in us:
+// split scan.  Whole scans over 5 bounces, 8 / 16 / 32 lanes, in us; binary nodes:
 //   rays    room             200k campus      5M city
 //   400     236 / 244 / 251  348 / 361 / 376  362 / 376 / 392
 //   3,200   259 / 266 / 269  408 / 413 / 423  435 / 446 / 457
@@ -389,8 +389,14 @@ static int graph_launch(rr_scene* s, ExecCtx* x, const ScanArgs& a, bool pattern
 //   6,000   271 / 274 / 270  453 / 452 / 444  478 / 481 / 482
 //   8,000   295 / 288 / 273  492 / 487 / 461  507 / 507 / 486
 // and in three ranges of 4,000 (12,000 rays) 320 / 307 / 302, 528 / 483 / 469,
-// 540 / 522 / 515: 16 lanes are never the best.
-static uint32_t query_lanes(uint64_t rays) { return rays <= 5120u ? 8u : 32u; }
+// 540 / 522 / 515: 16 lanes are never the best.  Wide nodes (a visit is the work
+// of eight lanes' visits, so fewer warps fill the issue slots):
+//   rays    room             200k campus      1M campus
+//   400     233 / 238 / 249  383 / 394 / 410  376 / 389 / 404
+//   1,600   255 / 256 / 260  422 / 423 / 426  410 / 413 / 419
+//   3,200   271 / 271 / 271  471 / 454 / 456  461 / 445 / 447
+//   4,800   282 / 271 / 275  537 / 492 / 483  517 / 479 / 474
+static uint32_t query_lanes(uint64_t rays, bool wide) { return rays <= (wide ? 2048u : 5120u) ? 8u : 32u; }
 
 int batch_enqueue(rr_scene* s, ExecCtx* x, const rr_pose* poses, const rr_sensor_params* ps, float* const* images,
                   uint32_t n, const DebugOut* dbg, cudaStream_t st, void* ws, const WsLayout& L, bool profile,
@@ -490,7 +496,7 @@ int batch_enqueue(rr_scene* s, ExecCtx* x, const rr_pose* poses, const rr_sensor
   a.defer_vis = (any_flags & RR_MULTIPATH) && maxb > 1 && !min_energy ? 1u : 0u;
   a.vis_list = (uint32_t*)(w + L.off_vis);
   const uint64_t in_flight = az_range ? (uint64_t)ps[0].n_azimuth * ps[0].rays_per_beam : rays;
-  a.lanes = cfg.trace_block == 64u && !(any_flags & RR_COUNT_TRAVERSAL) ? query_lanes(in_flight) : 32u;
+  a.lanes = cfg.trace_block == 64u && !(any_flags & RR_COUNT_TRAVERSAL) ? query_lanes(in_flight, wide) : 32u;
   a.refill = std::min(cfg.refill, a.lanes);
   a.rays[0] = (rr::RayRec*)(w + L.off_rays0);
   a.rays[1] = (rr::RayRec*)(w + L.off_rays1);
