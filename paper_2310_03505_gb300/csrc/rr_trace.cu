@@ -502,7 +502,6 @@ __device__ __forceinline__ void step_wide_node(Trav& s, uint2* stack, const Scan
   const uint32_t oct = s.oct, slot = (__ffs(bits) - 1u) ^ oct;
   bits &= bits - 1u;   // the lowest bit is a pending child's
   const uint32_t at = base + __popc((bits >> 8) & ((1u << slot) - 1u)), node = min(at, a.node_cap - 1u);
-  if (at >= a.node_cap) atomicOr(&a.ctr->error, kErrBvh);   // no build that reports success gets here
   if (bits & 0xFFu) stack[s.sp] = make_uint2(base, bits);
   s.sp += (bits & 0xFFu) ? 1 : 0;
   if (count) ++n_nodes;
@@ -511,6 +510,7 @@ __device__ __forceinline__ void step_wide_node(Trav& s, uint2* stack, const Scan
   const bool neg_x = id.x < 0.0f, neg_y = id.y < 0.0f, neg_z = id.z < 0.0f;
   const uint4* np = a.nodes + kWideNodeWords * (size_t)node;
   const uint4 w0 = __ldg(np), w1 = __ldg(np + 1), w2 = __ldg(np + 2), w3 = __ldg(np + 3), w4 = __ldg(np + 4);
+  if (at >= a.node_cap) atomicOr(&a.ctr->error, kErrBvh);   // no build that reports success gets here
   const float sx = __uint_as_float((w0.w & 0xFFu) << 23), sy = __uint_as_float(((w0.w >> 8) & 0xFFu) << 23),
               sz = __uint_as_float(((w0.w >> 16) & 0xFFu) << 23);
   // the node holds P - 2^23 s
