@@ -294,24 +294,28 @@ void ctx_free(ExecCtx* x) {
 
 using namespace rr_host;
 
-// what a finished build says of its grid (kCoarse), for the next one; true if that changes the nodes' form
-static bool note_coarse(rr_scene* s, const uint32_t* misc) {
-  const uint32_t coarse = misc[rr::kFrameWord + 3] != 0u ? 1u : 0u;
-  if (coarse == s->main.h_ctr->coarse) return false;
-  s->main.h_ctr->coarse = coarse;
-  if (cudaMemcpy(&s->main.d_ctr->coarse, &coarse, sizeof coarse, cudaMemcpyHostToDevice) != cudaSuccess)
-    cudaGetLastError();
-  return true;
+// what the build just queued says of its grid (kCoarse), for the next one;
+// *changed: that asks for the nodes' other form.  Waits for the stream.
+static cudaError_t note_coarse(rr_scene* s, cudaStream_t st, bool* changed) {
+  uint32_t coarse = 0;
+  cudaError_t e = build_status(s, st, false);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(&coarse, &s->main.d_ctr->coarse, sizeof coarse, cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  *changed = e == cudaSuccess && coarse != s->main.h_ctr->coarse;
+  if (e == cudaSuccess) s->main.h_ctr->coarse = coarse;
+  return e;
 }
 
 int rr_host::rebuild_bvh(rr_scene* s, cudaStream_t st) {
   if (s->nt == 0) return RR_OK;
-  uint32_t misc[rr::kMiscWords];
-  for (int pass = 0; pass < 2; ++pass) {   // again if the nodes' form has to change
+  uint32_t misc[8];
+  bool again = true;
+  for (int pass = 0; pass < 2 && again; ++pass) {   // again if the nodes' form has to change
     RR_CHECK_CUDA(build_lbvh(s, st, true), "rebuilding the BVH");
     RR_CHECK_CUDA(cudaMemcpyAsync(misc, s->d_misc, sizeof misc, cudaMemcpyDeviceToHost, st), "reading the build status");
-    RR_CHECK_CUDA(cudaStreamSynchronize(st), "rebuilding the BVH");
-    if (misc[6] || !note_coarse(s, misc)) break;
+    RR_CHECK_CUDA(note_coarse(s, st, &again), "rebuilding the BVH");
+    again = again && misc[6] == 0u;
   }
   if (misc[6] & rr::kErrTopBuild) return fail(RR_ERR_CUDA, "the SAH top of the BVH could not be built");
   if (misc[6]) return fail(RR_ERR_INVALID_ARG, "the scene's vertices are invalid");
@@ -319,15 +323,6 @@ int rr_host::rebuild_bvh(rr_scene* s, cudaStream_t st) {
   if (s->depth > (uint32_t)rr::kStack)
     return fail(RR_ERR_CAPACITY, "BVH depth " + std::to_string(s->depth) + " exceeds the traversal stack");
   return RR_OK;
-}
-
-// one-thread kernel folding the build status into the scan status word
-__global__ void k_fold_build_status(const uint32_t* misc, const uint32_t* wctr, ScanCounters* ctr) {
-  uint32_t e = 0;
-  if (misc[6] & ~rr::kErrTopBuild) e |= rr::kErrBadVertex;
-  if ((misc[6] & rr::kErrTopBuild) || wctr[4]) e |= rr::kErrBvh;
-  if (e) atomicOr(&ctr->error, e);
-  ctr->coarse = misc[rr::kFrameWord + 3] != 0u ? 1u : 0u;
 }
 
 extern "C" {
@@ -494,7 +489,7 @@ int rr_scene_create(const float* vertices, uint32_t n_vertices, const uint32_t* 
   cudaEventDestroy(e1);
   s->build_ms = ms;
   if (n_triangles) {
-    uint32_t misc[rr::kMiscWords];
+    uint32_t misc[8];
     e = cudaMemcpy(misc, s->d_misc, sizeof misc, cudaMemcpyDeviceToHost);
     if (e != cudaSuccess) return bail(cuda_fail(e, "reading the build status"));
     if (misc[6] & 1u) return bail(fail(RR_ERR_INVALID_ARG, "a triangle references a vertex index >= n_vertices"));
@@ -504,7 +499,9 @@ int rr_scene_create(const float* vertices, uint32_t n_vertices, const uint32_t* 
     s->depth = misc[7];
     if (s->depth > (uint32_t)rr::kStack)
       return bail(fail(RR_ERR_CAPACITY, "BVH depth " + std::to_string(s->depth) + " exceeds the traversal stack"));
-    if (note_coarse(s, misc))
+    bool again = false;
+    if ((e = note_coarse(s, st, &again)) != cudaSuccess) return bail(cuda_fail(e, "reading the build status"));
+    if (again)
       if (int rc = rebuild_bvh(s, st)) return bail(rc);
   }
   *out = s;
@@ -522,11 +519,7 @@ int rr_scene_update_vertices(rr_scene* s, const float* vertices) {
   prof_begin(s, RR_K_BUILD, st, &ev);
   RR_CHECK_CUDA(build_lbvh(s, st, false), "rebuilding the BVH");
   prof_end(s, ev, st);
-  if (s->nt) {
-    s->launches += 1;
-    k_fold_build_status<<<1, 1, 0, st>>>(s->d_misc, s->d_wctr, s->main.d_ctr);
-    RR_CHECK_CUDA(cudaGetLastError(), "status fold");
-  }
+  if (s->nt) RR_CHECK_CUDA(build_status(s, st, true), "status fold");
   return RR_OK;
 }
 

@@ -65,21 +65,11 @@ __device__ __forceinline__ void st_release_u32(uint32_t* p, uint32_t v) {
 // a1: validation, centroids and centroid bounds
 // misc[0..2] = ~encoded min xyz of the centroids, misc[3..5] = encoded max
 // xyz, misc[6] = error, misc[8..13] = the same bounds of the vertices (each a
-// maximum, so that all start from zero), misc[14..15] = sum over the triangles
-// with an extent of the float bits of their largest extent, without the last
-// 15 (piecewise linear in its logarithm, so the mean is near the geometric
-// one and a few huge triangles do not move it), misc[16] = their count
+// maximum, so that all start from zero)
 __global__ void k_ingest(const float* __restrict__ vtx, const uint32_t* __restrict__ idx,
                          const uint16_t* __restrict__ mat_id, uint32_t nv, uint32_t nt, uint32_t nm,
                          float4* __restrict__ centroid, uint32_t* __restrict__ misc) {
   __shared__ float s_lo[6][32], s_hi[6][32];
-  __shared__ unsigned long long s_size;
-  __shared__ uint32_t s_sized;
-  if (threadIdx.x == 0) {
-    s_size = 0ull;
-    s_sized = 0u;
-  }
-  uint32_t size = 0u, sized = 0u;   // a thread has at most some 3,500 of 2^30 triangles: size < 2^32
   float lo[6], hi[6];   // centroid, vertices
   for (int k = 0; k < 6; ++k) {
     lo[k] = INFINITY;
@@ -113,16 +103,10 @@ __global__ void k_ingest(const float* __restrict__ vtx, const uint32_t* __restri
         lo[3 + k] = fminf(lo[3 + k], vlo[k]);
         hi[3 + k] = fmaxf(hi[3 + k], vhi[k]);
       }
-      const float ext = fmaxf(fmaxf(vhi[0] - vlo[0], vhi[1] - vlo[1]), vhi[2] - vlo[2]);
-      size += __float_as_uint(ext) >> 15;
-      sized += ext > 0.0f ? 1u : 0u;
     }
     centroid[i] = make_float4(cen[0], cen[1], cen[2], 0.f);
   }
-  // warp then block reduction of the bounds and sizes
-  unsigned long long wsize = size;
-  for (int off = 16; off > 0; off >>= 1) wsize += __shfl_xor_sync(0xFFFFFFFFu, wsize, off);
-  sized = __reduce_add_sync(0xFFFFFFFFu, sized);
+  // warp then block reduction of the bounds
   for (int k = 0; k < 6; ++k) {
     for (int off = 16; off > 0; off >>= 1) {
       lo[k] = fminf(lo[k], __shfl_xor_sync(0xFFFFFFFFu, lo[k], off));
@@ -136,15 +120,6 @@ __global__ void k_ingest(const float* __restrict__ vtx, const uint32_t* __restri
       s_hi[k][warp] = hi[k];
     }
   __syncthreads();
-  if (lane == 0 && sized) {
-    atomicAdd(&s_size, wsize);
-    atomicAdd(&s_sized, sized);
-  }
-  __syncthreads();
-  if (threadIdx.x == 0 && s_sized) {
-    atomicAdd(reinterpret_cast<unsigned long long*>(misc + kSizeWord), s_size);
-    atomicAdd(&misc[kSizeWord + 2], s_sized);
-  }
   if (warp == 0) {
     for (int k = 0; k < 6; ++k) {
       float l = lane < nw ? s_lo[k][lane] : INFINITY, h = lane < nw ? s_hi[k][lane] : -INFINITY;
@@ -170,16 +145,6 @@ __device__ __forceinline__ uint32_t spread3(uint32_t v) {
   return v;
 }
 
-// Grid step (of its coarser half) over the mean triangle size above which the
-// binary nodes should hold float boxes.  Scans of 400 x 200 rays over the
-// repository's scenes (their own grids: 0.004 to 0.021) with one more triangle
-// below the ground that stretches the grid, grid / float boxes in us:
-//   200k campus  0.004  895 / 980   0.067  979 / 958    0.22 1,143 / 964   2.2  2,834 / 952   22  48,370 / 955
-//   1M campus    0.012  814 / 864   0.070  869 / 864    0.21   925 / 865   0.70 1,123 / 862
-//   5M city      0.021  970 / 1,089 0.061  1,017 / 1,089 0.18 1,101 / 1,090 0.61 1,276 / 1,090
-// (the coarser the grid, the more triangles share a cell: 3 to 770 tests a query).
-constexpr float kCoarse = 0.125f;
-
 // a2: code = x9 y9 z9 x8 y8 z8 ... x0 y0 z0 of the quantised centroid
 // also counts the first sort pass's digits per tile (hist0, zeroed before)
 // and lays the grid of the binary nodes over the vertex bounds
@@ -193,7 +158,6 @@ __global__ void k_morton(const float4* __restrict__ centroid, uint32_t* __restri
     // either side for the outward rounding.  The scale is at least 2^-11 of
     // the coordinates, so that rounding the base moves no bound out of range.
     float* fr = reinterpret_cast<float*>(misc + kFrameWord);
-    float widest = 0.0f;
     for (int k = 0; k < 3; ++k) {
       float lo = dec_f(~misc[8 + k]), hi = dec_f(misc[11 + k]);
       if (!(lo <= hi)) lo = hi = 0.0f;   // no valid triangle: the build is reported as failed
@@ -202,13 +166,8 @@ __global__ void k_morton(const float4* __restrict__ centroid, uint32_t* __restri
       fr[k] = lo - 0.501f * scale;
       fr[4 + k] = scale;
       fr[8 + k] = 1.0f / scale;   // for the nodes' codes
-      widest = fmaxf(widest, scale);
     }
-    const uint32_t sized = misc[kSizeWord + 2];
-    const unsigned long long size = *reinterpret_cast<const unsigned long long*>(misc + kSizeWord);
-    const float mean = sized ? __uint_as_float((uint32_t)(size / sized) << 15) : INFINITY;
-    fr[3] = 0x1p-15f * widest > kCoarse * mean ? 1.0f : 0.0f;
-    fr[7] = fr[11] = 0.0f;
+    fr[3] = fr[7] = fr[11] = 0.0f;
   }
   const float4 c = centroid[i];
   const float cc[3] = {c.x, c.y, c.z};
@@ -611,21 +570,17 @@ __device__ __forceinline__ uint32_t grid_hi(float x, float base, float inv) {
   return ((__float_as_uint(f) + 0xFFu) >> 8) & 0xFFFFu;
 }
 
-// binary node p: boxes b0, b1 (lo xyz, hi xyz) of its children c0, c1; far:
-// the second array of nodes with float boxes, or null for nodes on the grid
-__device__ __forceinline__ void write_node(uint4* __restrict__ nodes, uint4* __restrict__ far, size_t p,
-                                           const float* __restrict__ frame, const float* b0, const float* b1,
-                                           uint32_t c0, uint32_t c1) {
-  if (far != nullptr) {
-    const auto half = [p](uint4* q, const float* b, uint32_t r0, uint32_t r1) {
-      q += kNodeWords * p;
-      q[0] = make_uint4(__float_as_uint(b[0]), __float_as_uint(b[3]), __float_as_uint(b[1]), __float_as_uint(b[4]));
-      q[1] = make_uint4(__float_as_uint(b[2]), __float_as_uint(b[5]), r0, r1);
-    };
-    half(nodes, b0, c0, c1);
-    half(far, b1, 0u, 0u);
-    return;
-  }
+// binary node p with float boxes: one child's half, in one of the two arrays
+__device__ __forceinline__ void write_exact(uint4* __restrict__ nodes, size_t p, const float* b, uint32_t r0,
+                                            uint32_t r1) {
+  nodes[kNodeWords * p] =
+      make_uint4(__float_as_uint(b[0]), __float_as_uint(b[3]), __float_as_uint(b[1]), __float_as_uint(b[4]));
+  nodes[kNodeWords * p + 1] = make_uint4(__float_as_uint(b[2]), __float_as_uint(b[5]), r0, r1);
+}
+
+// binary node p: boxes b0, b1 (lo xyz, hi xyz) of its children c0, c1
+__device__ __forceinline__ void write_node(uint4* __restrict__ nodes, size_t p, const float* __restrict__ frame,
+                                           const float* b0, const float* b1, uint32_t c0, uint32_t c1) {
   uint32_t w[6];
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
@@ -646,7 +601,10 @@ __device__ __forceinline__ void write_node(uint4* __restrict__ nodes, uint4* __r
 // of its range) is merged through shared memory -- arrival counter and child
 // boxes -- so the bottom levels of every walk cost no L2 round trips; the
 // others through the global counters and nbox.
+// kExact: nodes with float boxes (far is their second array; apart, because the
+// choice inside costs 28 us of a rebuild of 5M triangles).
 constexpr int kRefitBlock = 256;
+template <bool kExact>
 __global__ void __launch_bounds__(kRefitBlock) k_refit(uint32_t n, const uint32_t* __restrict__ child,
                                                        const uint32_t* __restrict__ parent,
                                                        const uint2* __restrict__ range, uint32_t* __restrict__ visit,
@@ -695,7 +653,12 @@ __global__ void __launch_bounds__(kRefitBlock) k_refit(uint32_t n, const uint32_
       b0[k] = first_is_own ? own[k] : sb[k];
       b1[k] = first_is_own ? sb[k] : own[k];
     }
-    write_node(nodes, far, p, frame, b0, b1, c0, c1);
+    if (kExact) {
+      write_exact(nodes, p, b0, c0, c1);
+      write_exact(far, p, b1, 0u, 0u);
+    } else {
+      write_node(nodes, p, frame, b0, b1, c0, c1);
+    }
     float* bp = nbox + 6 * (size_t)p;
     for (int k = 0; k < 3; ++k) {
       own[k] = fminf(b0[k], b1[k]);
@@ -708,6 +671,62 @@ __global__ void __launch_bounds__(kRefitBlock) k_refit(uint32_t n, const uint32_
     cur = p;
     p = pp;
   }
+}
+
+// Grid step (of its coarser half) over the mean triangle size above which the
+// binary nodes should hold float boxes.  Scans of 400 x 200 rays over the
+// repository's scenes (their own grids: 0.004 to 0.021) with one more triangle
+// below the ground that stretches the grid, grid / float boxes in us:
+//   200k campus  0.004  895 / 980   0.067  979 / 958    0.22 1,143 / 964   2.2  2,834 / 952   22  48,370 / 955
+//   1M campus    0.012  814 / 864   0.070  869 / 864    0.21   925 / 865   0.70 1,123 / 862
+//   5M city      0.021  970 / 1,089 0.061  1,017 / 1,089 0.18 1,101 / 1,090 0.61 1,276 / 1,090
+// (the coarser the grid, the more triangles share a cell: 3 to 770 tests a query).
+constexpr float kCoarse = 0.125f;
+// The mean is taken over the largest extents of up to 256 triangles, one a
+// thread of k_build_status, evenly spaced in Morton order: of their float
+// bits, which are piecewise linear in the logarithm, so it is near the
+// geometric mean and a few huge triangles do not move it.  (All triangles in
+// the ingest: 6 us of a rebuild of 200k, 1,024 here 3 us.)
+constexpr int kStatusBlock = 256;
+
+// One block after a build: whether its grid is coarse, for the host (build_lbvh),
+// and, where asked for, its errors into the scan status word
+__global__ void __launch_bounds__(kStatusBlock) k_build_status(const uint32_t* __restrict__ misc,
+                                                               const uint32_t* __restrict__ wctr, uint32_t n,
+                                                               const float* __restrict__ nbox, bool errors,
+                                                               ScanCounters* __restrict__ ctr) {
+  __shared__ uint32_t s_size[kStatusBlock / 32], s_sized[kStatusBlock / 32];
+  const float* scale = reinterpret_cast<const float*>(misc + kFrameWord) + 4;
+  const float step = 0x1p-15f * fmaxf(fmaxf(scale[0], scale[1]), scale[2]);
+  const uint32_t err = errors ? misc[6] : 0u, wide_err = errors ? wctr[4] : 0u;
+  uint32_t size = 0u, sized = 0u;   // sums of at most 256 x 65,280
+  if (threadIdx.x < n) {
+    const size_t j = n <= kStatusBlock ? threadIdx.x : (uint64_t)threadIdx.x * n / kStatusBlock;
+    const float* b = nbox + 6 * ((size_t)n - 1 + j);
+    const float ext = fmaxf(fmaxf(b[3] - b[0], b[4] - b[1]), b[5] - b[2]);
+    if (ext > 0.0f && isfinite(ext)) {
+      size = __float_as_uint(ext) >> 15;
+      sized = 1u;
+    }
+  }
+  size = __reduce_add_sync(0xFFFFFFFFu, size);
+  sized = __reduce_add_sync(0xFFFFFFFFu, sized);
+  if ((threadIdx.x & 31u) == 0u) {
+    s_size[threadIdx.x >> 5] = size;
+    s_sized[threadIdx.x >> 5] = sized;
+  }
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  for (int w = 1; w < kStatusBlock / 32; ++w) {
+    size += s_size[w];
+    sized += s_sized[w];
+  }
+  const float mean = sized ? __uint_as_float(size / sized << 15) : INFINITY;
+  ctr->coarse = step > kCoarse * mean ? 1u : 0u;
+  uint32_t e = 0;
+  if (err & ~kErrTopBuild) e |= kErrBadVertex;
+  if ((err & kErrTopBuild) || wide_err) e |= kErrBvh;
+  if (e) atomicOr(&ctr->error, e);
 }
 
 // depth of every leaf (number of internal ancestors), maximum into misc[7]
@@ -1001,7 +1020,12 @@ __device__ Split warp_best_split(const uint32_t* bins, int lane) {
 // the node of a task: child boxes (lo xyz, hi xyz) and references
 __device__ __forceinline__ void write_top_node(const TopArgs& a, uint32_t slot, const float (&bx)[2][6],
                                                const uint32_t (&ref)[2]) {
-  write_node(a.nodes, a.far, slot, a.frame, bx[0], bx[1], ref[0], ref[1]);
+  if (a.far != nullptr) {
+    write_exact(a.nodes, slot, bx[0], ref[0], ref[1]);
+    write_exact(a.far, slot, bx[1], 0u, 0u);
+  } else {
+    write_node(a.nodes, slot, a.frame, bx[0], bx[1], ref[0], ref[1]);
+  }
   a.child[2 * slot] = ref[0];
   a.child[2 * slot + 1] = ref[1];
   for (int side = 0; side < 2; ++side) a.parent[node_slot(ref[side], a.n)] = slot;
@@ -2153,7 +2177,7 @@ cudaError_t build_lbvh(rr_scene* s, cudaStream_t st, bool with_depth) {
     else cudaGetLastError();
   }
   s->exact_nodes = s->main.h_ctr->coarse && s->d_far;
-  // bounds, error, depth and sizes start from zero
+  // bounds, error and depth start from zero
   RR_TRY(cudaMemsetAsync(s->d_misc, 0, kFrameWord * sizeof(uint32_t), st));
   if (n == 0) return cudaSuccess;
   const int B = 256;
@@ -2199,10 +2223,10 @@ cudaError_t build_lbvh(rr_scene* s, cudaStream_t st, bool with_depth) {
     k_karras<<<(n - 1 + B - 1) / B, B, 0, st>>>(s->d_keys[cur], (int)n, s->d_child, s->d_parent, s->d_visit,
                                                 s->d_range);
     RR_TRY(cudaGetLastError());
-    k_refit<<<(n + kRefitBlock - 1) / kRefitBlock, kRefitBlock, 0, st>>>(n, s->d_child, s->d_parent, s->d_range,
-                                                                           s->d_visit, s->d_nbox, s->d_nodes,
-                                                                           s->exact_nodes ? s->d_far : nullptr,
-                                                                           reinterpret_cast<const float*>(s->d_misc + kFrameWord));
+    auto* refit = s->exact_nodes ? k_refit<true> : k_refit<false>;
+    refit<<<(n + kRefitBlock - 1) / kRefitBlock, kRefitBlock, 0, st>>>(n, s->d_child, s->d_parent, s->d_range,
+                                                                         s->d_visit, s->d_nbox, s->d_nodes, s->d_far,
+                                                                         reinterpret_cast<const float*>(s->d_misc + kFrameWord));
     RR_TRY(cudaGetLastError());
     if (sah_top) RR_TRY(build_sah_top(s, st));
     if (with_depth) {
@@ -2216,6 +2240,12 @@ cudaError_t build_lbvh(rr_scene* s, cudaStream_t st, bool with_depth) {
   }
   s->wide_stale = true;   // the 8-wide BVH is collapsed when a scan first needs it
   return cudaSuccess;
+}
+
+cudaError_t build_status(rr_scene* s, cudaStream_t st, bool errors) {
+  s->launches += 1u;
+  k_build_status<<<1, kStatusBlock, 0, st>>>(s->d_misc, s->d_wctr, s->nt, s->d_nbox, errors, s->main.d_ctr);
+  return cudaGetLastError();
 }
 
 // a6: the 8-wide quantised BVH, collapsed from the current binary LBVH

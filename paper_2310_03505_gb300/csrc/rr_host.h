@@ -115,7 +115,7 @@ struct rr_scene {
   uint32_t* d_child = nullptr;     // [T-1][2]
   float* d_nbox = nullptr;         // [2T-1][6]
   uint32_t* d_visit = nullptr;     // [T-1]
-  uint32_t* d_misc = nullptr;      // [kMiscWords]: bounds (encoded), error bits, depth, sizes, node grid
+  uint32_t* d_misc = nullptr;      // [kMiscWords]: bounds (encoded), error bits, depth, node grid
   uint2* d_range = nullptr;        // [T-1] leaf range (first, last) of every internal node
   // SAH top over the LBVH's subtrees (allocated with the first such build)
   uint32_t* d_cl_at = nullptr;     // [T] cluster root reference at the cluster's first leaf, else kNone
@@ -156,6 +156,7 @@ namespace rr_host {
 
 // rr_build.cu
 cudaError_t build_alloc(rr_scene* s);
+cudaError_t build_status(rr_scene* s, cudaStream_t st, bool errors);   // after a build: the grid's state and, if asked for, errors into the main context's counters
 cudaError_t build_lbvh(rr_scene* s, cudaStream_t st, bool with_depth);   // a1..a5 on s->d_vtx; counts its launches
 cudaError_t build_materials(rr_scene* s, cudaStream_t st);
 cudaError_t build_wide(rr_scene* s, cudaStream_t st);      // a6, stream ordered after the LBVH

@@ -94,7 +94,7 @@ struct ScanCounters {
   uint32_t vis_ticket[RR_MAX_BOUNCES];
   uint32_t need_rays, need_recs;           // largest request seen (overflow report)
   uint32_t error;                          // sticky kErr* bits
-  uint32_t coarse;                         // the scene's grid is too coarse (kCoarse), as of its last build
+  uint32_t coarse;                         // the scene's grid is coarse beside its triangles (kCoarse), as of its last build
   unsigned long long stat_closest, stat_anyhit, stat_returns, stat_scans;
   unsigned long long stat_nodes, stat_tris;
   unsigned long long stat_nodes_any, stat_tris_any;
@@ -132,11 +132,9 @@ constexpr int kWideNodeWords = 5;
 // place of a second array, each as (lo x, hi x, lo y, hi y) (lo z, hi z,
 // child0, child1), the references with child 0 only.
 constexpr int kNodeWords = 2;
-// The grid of a scene's binary nodes, three float4: (base x, y, z, f), (scale x, y, z, 0), (1 / scale, 0),
-// f: 1 where it is too coarse
-constexpr int kFrameWord = 20;        // its place in the build status words (rr_scene::d_misc)
-constexpr int kSizeWord = 14;         // sum (64 bits) and count of the triangles' sizes (k_ingest)
-constexpr int kMiscWords = 32;        // 0..5 centroid bounds, 6 error bits, 7 depth, 8..13 vertex bounds, 14..16 sizes, 20..31 the frame
+// The grid of a scene's binary nodes, three float4: (base x, y, z, 0), (scale x, y, z, 0), (1 / scale, 0)
+constexpr int kFrameWord = 16;        // its place in the build status words (rr_scene::d_misc)
+constexpr int kMiscWords = 28;        // 0..5 centroid bounds, 6 error bits, 7 depth, 8..13 vertex bounds, 16..27 the frame
 
 // Return record key: global image column (scan's first column + azimuth)
 // and range bin.  Records of one bounce are in column order.
