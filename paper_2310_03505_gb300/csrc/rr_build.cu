@@ -75,9 +75,10 @@ __global__ void k_ingest(const float* __restrict__ vtx, const uint32_t* __restri
     lo[k] = INFINITY;
     hi[k] = -INFINITY;
   }
-  // a few blocks per SM, each over many triangles: the bounds end in twelve
-  // atomics per block on the same words (5M triangles: 58 us, 201 with a block per
-  // 256 triangles)
+  // a few blocks per SM, each over several triangles a thread: the bounds end
+  // in twelve atomics per block on the same words (5M triangles: 58 us, 201 with
+  // a block per 256 triangles; a rebuild of 200k: 176 us with four triangles a
+  // thread, 180 with one; with fewer blocks than SMs 50k get 2 us slower)
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < nt; i += gridDim.x * blockDim.x) {
     uint32_t err = 0;
     float vlo[3] = {0.f, 0.f, 0.f}, vhi[3] = {0.f, 0.f, 0.f};
@@ -2185,8 +2186,9 @@ cudaError_t build_lbvh(rr_scene* s, cudaStream_t st, bool with_depth) {
   const bool sah_top = s->cfg.bvh_build == RR_BVH_SAH_TOP && n > kClusterMax;
   s->launches += ((n > 1) ? (with_depth ? 14u : 13u) : 11u) + (sah_top ? 6u : 0u) +
                  ((size_t)256 * s->sort_tiles > kScanSingleMax ? 8u : 0u);   // 3 launches per pass's counter scan
-  k_ingest<<<std::min<uint32_t>(g, 8u * (uint32_t)num_sms()), B, 0, st>>>(s->d_vtx, s->d_idx, s->d_mat_id, s->nv, n,
-                                                                             s->nm, s->d_centroid, s->d_misc);
+  const uint32_t sms = (uint32_t)num_sms();
+  k_ingest<<<std::min(std::min(g, 8u * sms), std::max(sms, g / 4u)), B, 0, st>>>(s->d_vtx, s->d_idx, s->d_mat_id, s->nv,
+                                                                                  n, s->nm, s->d_centroid, s->d_misc);
   RR_TRY(cudaGetLastError());
   // the four passes' digit counts per tile, zeroed, counted as each pass's input is written
   const size_t hist_words = (size_t)256 * s->sort_tiles;
