@@ -390,7 +390,7 @@ int rr_scan_batch_async(rr_scene* scene, uint32_t n, const rr_pose* poses, const
    refill_threshold     the query kernels keep their lanes busy by handing a
                         warp's idle lanes new queries once at least this many
                         of its 32 lanes are idle (1..32; 0 = 16).  Scans of at
-                        most 5,120 initial rays (2,048 over the wide nodes) in
+                        most 4,608 initial rays (2,048 over the wide nodes) in
                         64-thread blocks use 8 lanes a warp: there 8 and more
                         wait until all are idle
    workspace_limit      bytes of scan workspace; a launch sequence is sized

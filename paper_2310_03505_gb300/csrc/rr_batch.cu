@@ -386,17 +386,19 @@ static int graph_launch(rr_scene* s, ExecCtx* x, const ScanArgs& a, bool pattern
 //   400     236 / 244 / 251  348 / 361 / 376  362 / 376 / 392
 //   3,200   259 / 266 / 269  408 / 413 / 423  435 / 446 / 457
 //   4,000   258 / 261 / 269  424 / 428 / 436  445 / 452 / 456
+//   4,400   261 / 260 / 268  429 / 428 / 432  (1M campus 385 / 386 / 382)
+//   4,800   275 / 272 / 274  441 / 439 / 443  (1M campus 401 / 401 / 394)
 //   6,000   271 / 274 / 270  453 / 452 / 444  478 / 481 / 482
 //   8,000   295 / 288 / 273  492 / 487 / 461  507 / 507 / 486
 // and in three ranges of 4,000 (12,000 rays) 320 / 307 / 302, 528 / 483 / 469,
-// 540 / 522 / 515: 16 lanes are never the best.  Wide nodes (a visit is the work
-// of eight lanes' visits, so fewer warps fill the issue slots):
+// 540 / 522 / 515: 16 lanes gain nothing over the better of the two.  Wide nodes (a
+// visit is the work of eight binary ones, so fewer warps fill the issue slots):
 //   rays    room             200k campus      1M campus
 //   400     233 / 238 / 249  383 / 394 / 410  376 / 389 / 404
 //   1,600   255 / 256 / 260  422 / 423 / 426  410 / 413 / 419
 //   3,200   271 / 271 / 271  471 / 454 / 456  461 / 445 / 447
 //   4,800   282 / 271 / 275  537 / 492 / 483  517 / 479 / 474
-static uint32_t query_lanes(uint64_t rays, bool wide) { return rays <= (wide ? 2048u : 5120u) ? 8u : 32u; }
+static uint32_t query_lanes(uint64_t rays, bool wide) { return rays <= (wide ? 2048u : 4608u) ? 8u : 32u; }
 
 int batch_enqueue(rr_scene* s, ExecCtx* x, const rr_pose* poses, const rr_sensor_params* ps, float* const* images,
                   uint32_t n, const DebugOut* dbg, cudaStream_t st, void* ws, const WsLayout& L, bool profile,
@@ -558,15 +560,18 @@ int batch_run(rr_scene* s, ExecCtx* x, const rr_pose* poses, const rr_sensor_par
 // Whether a scan runs whole although the default would split it.  The ranges
 // overlap each other's slow queries, which pays once a bounce lasts well
 // beyond its launches: with few rays, or in a scene of few triangles (short
-// queries), the extra launches and the joins cost more.  Measured, split in 3
-// against whole: tiny room 3,200 rays 217 / 183 us and 40,000 rays 320 / 277;
-// 200k-triangle campus 12,000 rays 596 / 550, 24,000 rays 669 / 693, 40,000
-// rays 789 / 868; 5M-triangle city 24,000 rays 1,119 / 1,251.  The limit
+// queries), the extra launches and the joins cost more.  Measured over 5
+// bounces, split in 3 against whole, in us: room 3,200 rays 280 / 269, 16,000
+// 307 / 293, 40,000 371 / 344, 48,000 390 / 392, 64,000 434 / 454 (8-wide nodes
+// 32,000 387 / 386, 40,000 415 / 410, 48,000 447 / 462); campus of 50k and 200k, 1M
+// and city within 3 % of each other from 6,400 to 20,000 rays (campus 16,000 492 /
+// 504, city 545 / 544; 8-wide 589 / 605), then campus 1M 32,000 523 / 579, 64,000 736 /
+// 814.  The limit
 // counts per range, so a scan whose whole ray tree does not fit it stays split:
 // its ranges may hold what the whole would have to drop.
 static bool scan_whole(const rr_scene* s, const rr_sensor_params* p) {
   const uint64_t rays = (uint64_t)p->n_azimuth * p->rays_per_beam;
-  if (rays >= (1u << 14) && (s->nt >= (1u << 13) || rays >= (1u << 16))) return false;
+  if (rays >= (1u << 14) && (s->nt >= (1u << 13) || rays > 40960u)) return false;
   return !plan_workspace(p, 1, s->cfg.ws_limit, nullptr, s->cfg.order == RR_ORDER_CELL_OCTANT).clamped;
 }
 

@@ -339,8 +339,8 @@ def test_split_streams_default_and_explicit(tiny_scene):
             rr.rr_scene_destroy(h)
 
 
-# 5,120 and 5,121 rays, 2,048 and 2,049: the rule's lines
-@pytest.mark.parametrize("n_az,rays", [(1, 1), (400, 2), (320, 16), (569, 9), (256, 8), (683, 3)])
+# 4,608 and 4,609 rays, 2,048 and 2,049: the rule's lines
+@pytest.mark.parametrize("n_az,rays", [(1, 1), (400, 2), (288, 16), (419, 11), (256, 8), (683, 3)])
 @pytest.mark.parametrize("fmt", [rr.RR_NODES_BINARY, rr.RR_NODES_WIDE8])
 @pytest.mark.parametrize("cut", [0.0, 1e-7])   # visibility after and before the shading
 def test_few_lanes_equal_whole_warps(tiny_scene, n_az, rays, fmt, cut):
