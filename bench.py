@@ -742,14 +742,15 @@ def main():
                        step_bvh=args.step_bvh, node_format=args.node_format, ws_limit_gb=args.workspace_limit_gb,
                        e2e=not args.no_e2e, scan_only=not args.no_scan_only, clocks=rank == 0,
                        order=args.query_order)
-    campus_note = ("cache-resident: the campus BVH and triangles (~22 MB) stay in L2, so the algorithmic bytes "
+    campus_note = ("cache-resident: the campus BVH and triangles (~16 MB) stay in L2, so the algorithmic bytes "
                    "come from L1/L2 and the launches are bound by the latency of dependent node fetches, not by HBM")
     rl = roofline(head, peak, peak_kind, profile_counters("query_kernel_campus_ncu"), l2_peak, "latency",
                   campus_note) if args.no_large else \
         roofline(head, peak, peak_kind, profile_counters("query_kernel_city_ncu"), l2_peak, "latency",
-                  "the city's BVH and triangles (~0.56 GB) exceed the 129 MB L2, yet the dependent node fetches "
-                  "are served by L1 (79-81 % hit) and L2 (77-79 %): the kernel is bound by their latency, with L1 "
-                  "throughput the nearest limit (53-74 % of peak) and DRAM about 3 %.  achieved counts the "
+                  "the city's BVH and triangles (~0.40 GB) exceed the 129 MB L2, yet the dependent node fetches "
+                  "are served by L1 and L2 (87-89 % and 53-66 % hits on a 1M-triangle scene): the kernel is bound "
+                  "by their latency and, with 62-71 % of the issue slots taken there, by its instructions; DRAM "
+                  "carries about 2 %.  achieved counts the "
                   "algorithmic node/triangle/record bytes of a launch over its CUDA-event duration (the launches "
                   "of the 3 azimuth ranges and the previous bounce's visibility queries overlap them), against the HBM copy "
                   "peak; per_step divides a step's closest-hit bytes by the step time; dram_gbs and "
