@@ -68,3 +68,28 @@ def test_medium_full_scan_properties(medium):
     assert img.sum() > 0.5 * tal[..., 0].sum()
     st = rr.rr_scene_stats(h)
     assert st["closest_queries"] > 0
+
+
+@pytest.mark.parametrize("cut", [0.0, 1e-7])
+@pytest.mark.parametrize("split,rays", [(0, 200), (1, 200), (1, 100)])   # shading tiles of 256, 512 and 256 rays
+def test_medium_plain_scan_equals_the_debug_scan(medium, split, rays, cut):
+    """The comparisons above go through the debug dump, which has a shading
+    kernel of its own; a plain scan's image (both tile sizes, visibility after
+    and before the shading) agrees with the dump's up to the rounding of the
+    energies and of the bin sums."""
+    import torch
+    sc, pz, params, h = medium
+    p = scenes.sensor(**{**params, "rays_per_beam": rays, "min_energy": cut, "scan_id": 31})
+    ref, _, _ = P.gpu_debug(h, pz, p)
+    out = torch.zeros(p["n_azimuth"], p["n_bins"], device="cuda")
+    saved = rr.rr_batch_config_get(h)
+    try:
+        rr.rr_batch_config_set(h, split_streams=split)
+        rr.rr_scan(h, pz, p, out)
+    finally:
+        rr.rr_batch_config_set(h, **saved)
+    img = out.cpu().numpy()
+    assert np.count_nonzero(ref) > 10_000
+    # a few hundred roundings of 2^-24 relative to an energy, of which a pixel holds several
+    assert np.max(np.abs(img - ref)) <= 1e-5 * ref.max()
+    assert abs(img.sum(dtype=np.float64) - ref.sum()) <= 1e-5 * ref.sum()
